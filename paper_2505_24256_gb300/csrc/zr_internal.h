@@ -226,13 +226,9 @@ zr_status check_recon_args(zr_ctx* ctx, const zr_blackbox* bb, const zr_recon_pa
 // balanced step pieces (zr_balance.cu)
 void launch_probe_points(int64_t T, int S, int nv, int k, int offset, const uint64_t* y, const uint64_t* cs,
                          const uint64_t* z, const Mod& M, uint64_t* pts, cudaStream_t st);
-void launch_ratio(int64_t T, int S, const uint64_t* Nv, const uint64_t* Dv, int64_t ld, const Mod& M, uint64_t* pre,
-                  uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st);
-size_t thiele_scratch_words(int64_t Tmax, int n);
-void launch_thiele_balance(int64_t Tmax, int n, const uint64_t* xs, const uint64_t* fvals, int64_t ldf,
-                           const uint64_t* dprev, int dN, int dD, int64_t TN, int64_t TD, uint64_t* scratch,
-                           const Mod& M, uint64_t* bN, int64_t ldN, uint64_t* bD, int64_t ldD, uint32_t* status,
-                           cudaStream_t st);
+void launch_thiele_balance(int64_t Tmax, int n, const uint64_t* xs, const uint64_t* fvals, const uint64_t* fdens,
+                           int64_t ldf, const uint64_t* dprev, int dN, int dD, int64_t TN, int64_t TD, const Mod& M,
+                           uint64_t* bN, int64_t ldN, uint64_t* bD, int64_t ldD, uint32_t* status, cudaStream_t st);
 void launch_normalise(int64_t n1, uint64_t* a1, int64_t n2, uint64_t* a2, const uint64_t* pivot, uint64_t* tmp,
                       const Mod& M, uint32_t* status, cudaStream_t st);
 // kernels used by the reconstruction driver

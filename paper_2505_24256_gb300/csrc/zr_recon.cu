@@ -385,27 +385,17 @@ zr_status Recon::step0_rational() {
     std::vector<uint64_t> pts = step0_points(nv_, Sf, cs_.data(), z_.data());
     if ((r = upload(d_pts_, pts.data(), pts.size() * 8))) return r;
     if ((r = upload(d_cs_, cs_.data(), cs_.size() * 8))) return r;
-    cudaError_t e = d_vals_.ensure(8 * (size_t)Sf * 4 + 8 * (size_t)(dN + dD + 2));
+    cudaError_t e = d_vals_.ensure(8 * (size_t)Sf * 2 + 8 * (size_t)(dN + dD + 2));
     if (e != cudaSuccess) return cuda_err(ctx_, e, "values");
-    uint64_t* nvls = d_vals_.as<uint64_t>();
+    uint64_t* nvls = d_vals_.as<uint64_t>();      // N, or the caller's N / D
     uint64_t* dvls = nvls + Sf;
-    uint64_t* pre = dvls + Sf;
-    uint64_t* f = pre + Sf;
-    uint64_t* nval = f + Sf;
+    uint64_t* nval = dvls + Sf;
     uint64_t* dval = nval + (dN + 1);
-    if (callback_) {
-      r = eval_at(fN_, Sf, d_pts_.as<uint64_t>(), f);     // the caller's N / D
-    } else {
-      if (!(r = eval_at(fN_, Sf, d_pts_.as<uint64_t>(), nvls)) && !(r = eval_at(fD_, Sf, d_pts_.as<uint64_t>(), dvls))) {
-        launch_ratio(1, Sf, nvls, dvls, 1, M_, pre, f, 1, ctx_->d_status_call, st_);
-        r = sync_status();
-      }
-    }
+    r = eval_at(fN_, Sf, d_pts_.as<uint64_t>(), nvls);
+    if (!r && !callback_) r = eval_at(fD_, Sf, d_pts_.as<uint64_t>(), dvls);
     if (!r) {
-      e = persist_.ensure(8 * thiele_scratch_words(1, Sf) + 256);
-      if (e != cudaSuccess) return cuda_err(ctx_, e, "thiele scratch");
-      launch_thiele_balance(1, Sf, d_cs_.as<uint64_t>(), f, 1, one_.as<uint64_t>(), dN, dD, 1, 1,
-                            persist_.as<uint64_t>(), M_, nval, 1, dval, 1, ctx_->d_status_call, st_);
+      launch_thiele_balance(1, Sf, d_cs_.as<uint64_t>(), nvls, callback_ ? nullptr : dvls, 1, one_.as<uint64_t>(), dN,
+                            dD, 1, 1, M_, nval, 1, dval, 1, ctx_->d_status_call, st_);
       r = sync_status();
     }
     if ((r == ZR_ERR_POLE || r == ZR_ERR_UNLUCKY) && attempt_ + 1 < kMaxAttempts) {
@@ -510,20 +500,18 @@ zr_status Recon::prepare(std::vector<BatchItem>& items, uint32_t* d_status, int6
     if (r) return fail(r);
     const int64_t TN = curN_.T, TD = curD_.T, Tmax = std::max(TN, TD);
     if (Tmax == 0) break;
-    // f = N/D at (y^(i+off), c_s, z)
-    cudaError_t e = fv_.ensure(8 * (size_t)Sf * Tmax * 4);
+    // f = N/D at (y^(i+off), c_s, z): the pair, or the caller's values
+    cudaError_t e = fv_.ensure(8 * (size_t)Sf * Tmax * (callback_ ? 1 : 2));
     if (e != cudaSuccess) return fail(cuda_err(ctx_, e, "rational probes"));
     uint64_t* nvls = fv_.as<uint64_t>();
-    uint64_t* dvls = nvls + (size_t)Sf * Tmax;
-    uint64_t* pre = dvls + (size_t)Sf * Tmax;
-    uint64_t* f = pre + (size_t)Sf * Tmax;
+    uint64_t* dvls = callback_ ? nullptr : nvls + (size_t)Sf * Tmax;
     if (callback_) {
       // f = N/D from the caller at the probe points
       e = d_ppts_.ensure(8 * (size_t)Sf * Tmax * nv_);
       if (e != cudaSuccess) return fail(cuda_err(ctx_, e, "probe points"));
       launch_probe_points(Tmax, Sf, nv_, k, offset_, d_y_.as<uint64_t>(), d_cs_.as<uint64_t>(), d_z_.as<uint64_t>(),
                           M_, d_ppts_.as<uint64_t>(), st_);
-      r = eval_at(fN_, (int64_t)Sf * Tmax, d_ppts_.as<uint64_t>(), f);
+      r = eval_at(fN_, (int64_t)Sf * Tmax, d_ppts_.as<uint64_t>(), nvls);
       if (r && r != ZR_ERR_POLE) return fail(r);
     } else {
       zr_poly nv_p = fN_.view(), dv_p = fD_.view();
@@ -533,14 +521,11 @@ zr_status Recon::prepare(std::vector<BatchItem>& items, uint32_t* d_status, int6
         r = probes_impl(ctx_, &dv_p, k, d_y_.as<uint64_t>(), Sf, d_cs_.as<uint64_t>(), d_z_.as<uint64_t>(), Tmax,
                         offset_, dvls, Tmax, ctx_->d_status_call, st_);
       if (r) return fail(r);
-      launch_ratio(Tmax, Sf, nvls, dvls, Tmax, M_, pre, f, Tmax, ctx_->d_status_call, st_);
-      r = sync_status();
     }
     if (!r) {
       // D' at the probes, Thiele per probe, balancing
       const size_t w_dprev = (size_t)Tmax, w_bN = (size_t)SN * (TN ? TN : 1), w_bD = (size_t)SD * (TD ? TD : 1);
-      const size_t w_th = thiele_scratch_words(Tmax, Sf);
-      e = persist_.ensure(8 * (w_dprev + w_bN + w_bD + w_th) + 256);
+      e = persist_.ensure(8 * (w_dprev + w_bN + w_bD) + 256);
       if (e == cudaSuccess) e = ones_.ensure(8 * (size_t)nv_);
       if (e != cudaSuccess) return fail(cuda_err(ctx_, e, "balanced buffers"));
       {
@@ -552,7 +537,6 @@ zr_status Recon::prepare(std::vector<BatchItem>& items, uint32_t* d_status, int6
       uint64_t* dprev = persist_.as<uint64_t>();
       uint64_t* bN = dprev + w_dprev;
       uint64_t* bD = bN + w_bN;
-      uint64_t* th = bD + w_bD;
       zr_poly dsk = curD_.view();
       if (TD > 0)
         r = probes_impl(ctx_, &dsk, k, d_y_.as<uint64_t>(), 1, ones_.as<uint64_t>(), ones_.as<uint64_t>(), Tmax,
@@ -560,8 +544,8 @@ zr_status Recon::prepare(std::vector<BatchItem>& items, uint32_t* d_status, int6
       else
         cudaMemsetAsync(dprev, 0, 8 * Tmax, st_);
       if (r) return fail(r);
-      launch_thiele_balance(Tmax, Sf, d_cs_.as<uint64_t>(), f, Tmax, dprev, dN, dD, TN, TD, th, M_, bN, TN ? TN : 1, bD,
-                            TD ? TD : 1, ctx_->d_status_call, st_);
+      launch_thiele_balance(Tmax, Sf, d_cs_.as<uint64_t>(), nvls, dvls, Tmax, dprev, dN, dD, TN, TD, M_, bN,
+                            TN ? TN : 1, bD, TD ? TD : 1, ctx_->d_status_call, st_);
       r = sync_status();
       if (!r) {
         r = step_entry(curN_, SN, bN, TN ? TN : 1, nextN_, d_status, d_counts, items);
@@ -778,8 +762,7 @@ extern "C" zr_status zr_zippel_step_balanced(zr_ctx* ctx, const zr_poly* skelN, 
   DBuf persist, ones;
   persist.s = ones.s = st;   // allocated and freed in the order of the call's stream
   const size_t w_dprev = (size_t)Tmax, w_bN = (size_t)SN * (TN ? TN : 1), w_bD = (size_t)SD * (TD ? TD : 1);
-  const size_t w_th = thiele_scratch_words(Tmax, Sf);
-  cudaError_t e = persist.ensure(8 * (w_dprev + w_bN + w_bD + w_th) + 256);
+  cudaError_t e = persist.ensure(8 * (w_dprev + w_bN + w_bD) + 256);
   if (e == cudaSuccess) e = ones.ensure(8 * (size_t)nv);
   if (e == cudaSuccess) {
     const std::vector<uint64_t> h(nv, 1);
@@ -790,7 +773,6 @@ extern "C" zr_status zr_zippel_step_balanced(zr_ctx* ctx, const zr_poly* skelN, 
   uint64_t* dprev = persist.as<uint64_t>();
   uint64_t* bN = dprev + w_dprev;
   uint64_t* bD = bN + w_bN;
-  uint64_t* th = bD + w_bD;
   zr_status r = ZR_OK;
   if (TD > 0) {
     zr_poly dsk = *skelD;
@@ -800,7 +782,7 @@ extern "C" zr_status zr_zippel_step_balanced(zr_ctx* ctx, const zr_poly* skelN, 
     cudaMemsetAsync(dprev, 0, 8 * Tmax, st);
   }
   if (r) return r;
-  launch_thiele_balance(Tmax, Sf, samples, fvals, ldf, dprev, dN, dD, TN, TD, th, ctx->M, bN, TN ? TN : 1, bD,
+  launch_thiele_balance(Tmax, Sf, samples, fvals, nullptr, ldf, dprev, dN, dD, TN, TD, ctx->M, bN, TN ? TN : 1, bD,
                         TD ? TD : 1, ctx->d_status_call, st);
   // the numerator and denominator steps share one batch of launches
   BatchItem items[2];
