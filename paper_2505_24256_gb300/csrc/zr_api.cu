@@ -451,19 +451,35 @@ bool use_fast_solve(const zr_ctx* ctx, int64_t T, int S, int batch_n) {
 }  // namespace zr
 
 // The automatic choice of evaluator for T probes per sample of a function
-// of Tf terms and S samples.  Measured on GB300 (Tf = T): the matrix-vector
-// evaluator costs about S T Tf 5e-10 ms + 0.15 ms, the transposed tree 0.36
-// to 1.3 ms from T = 2048 to 16384; they cross near T = 7800 (S = 21),
-// 12500 (S = 5) and 14000 (S = 1), which T Tf (S + 8) >= 1.8e9 follows.
-static constexpr double kFastProbeCross = 1.8e9;
+// of Tf terms and S samples.  Measured on GB300 (Tf = T, whole call): the
+// transposed tree overtakes the product on the tensor cores near T = 105000
+// (S = 1), 50000 (5), 38000 (11), 29000 (21) and 20000 (42), which S T Tf >=
+// 1.5e10 follows (at T = 16000, S = 21: 0.74 against 1.23 ms; at 64000: 9.4
+// against 3.3 ms).
+static constexpr double kFastProbeCross = 1.5e10;
 static constexpr int64_t kFastProbeFloorT = 4096;
+// The tensor cores overtake the integer ring kernel near T = Tf = 2400 (S =
+// 1), 1900 (5), 1450 (11) and 1200 (21), which T min(T, Tf) (S + 4) >= 3.3e7
+// follows (T = 3000, S = 11: 0.089 against 0.132 ms; T = 1000: 0.074 against
+// 0.064 ms; a step asks for as many probes as the function has groups, so more
+// terms than probes mean groups of several terms).  Packing a group's 128 powers costs what the ring kernel takes for
+// (S + 4) T near 2000 (T = 300, Tf = 30000: 0.124 against 0.136 ms at S = 1),
+// so fewer products per group stay there; so do groups past kTcProbeMaxTf,
+// whose packed powers (2 KB each) would hold more than half a gigabyte.
+static constexpr double kTcProbeCross = 3.3e7;
+static constexpr double kTcProbeFloor = 2000;
+static constexpr int64_t kTcProbeMaxTf = 1ll << 18;
 
 namespace zr {
 bool use_fast_probes(const zr_ctx* ctx, int64_t T, int64_t Tf, int S) {
   if (T < 1 || Tf < 1 || T > kFastMaxT || S > kFastProbeMaxS || ctx->solve_method == 1) return false;
   if (ctx->solve_method == 2) return true;
   if (ctx->fast_min_T > 0) return T >= ctx->fast_min_T && Tf >= ctx->fast_min_T;
-  return T >= kFastProbeFloorT && Tf >= kFastProbeFloorT && (double)T * (double)Tf * (double)(S + 8) >= kFastProbeCross;
+  return T >= kFastProbeFloorT && Tf >= kFastProbeFloorT && (double)T * (double)Tf * (double)S >= kFastProbeCross;
+}
+bool use_tc_probes(int64_t T, int64_t Tf, int S) {
+  const double col = (double)T * (double)(S + 4);
+  return Tf <= kTcProbeMaxTf && col >= kTcProbeFloor && col * (double)std::min(T, Tf) >= kTcProbeCross;
 }
 }  // namespace zr
 
@@ -471,7 +487,8 @@ bool use_fast_probes(const zr_ctx* ctx, int64_t T, int64_t Tf, int S) {
 // second on GB300).  The O(T^2) solve does S T^2 + 2.5 T^2; the fast one was
 // measured at 25 ms for T = 2^20, S = 9 and about 0.5 ms at small T, which
 // 8 (S + 6) T log2(T)^2 + 1e9 follows.  The matrix-vector evaluator does
-// S T Tf; the transposed tree is weighted like the fast solve on max(T, Tf).
+// S T Tf, at a quarter of the weight on the tensor cores (8e12 to 9e12 per
+// second); the transposed tree is weighted like the fast solve on max(T, Tf).
 namespace zr {
 static double fast_work(double n, int S) {
   const double l = std::log2(std::max(n, 2.0));
@@ -483,8 +500,8 @@ double solve_work(const zr_ctx* ctx, int64_t T, int S) {
 }
 double probe_work(const zr_ctx* ctx, int64_t T, int S, int64_t Tf) {
   if (T <= 0 || Tf <= 0) return 0;
-  return use_fast_probes(ctx, T, Tf, S) ? fast_work((double)std::max(T, Tf), S)
-                                        : (double)S * (double)T * (double)Tf;
+  if (use_fast_probes(ctx, T, Tf, S)) return fast_work((double)std::max(T, Tf), S);
+  return (double)S * (double)T * (double)Tf * (use_tc_probes(T, Tf, S) ? 0.25 : 1.0);
 }
 }  // namespace zr
 

@@ -466,9 +466,12 @@ __global__ void __launch_bounds__(EvalRingCfg<CG, G>::NT, EvalRingCfg<CG, G>::MI
   }
 }
 
-__global__ void k_eval_combine(int64_t T, int S, int gsplit, const uint64_t* __restrict__ partial, Mod M,
-                               uint64_t* __restrict__ out, int64_t ldo) {
+// out = sum of the group splits' partial sums (with Gdev: of the splits the
+// tensor-core kernel used)
+__global__ void k_eval_combine(int64_t T, int S, int gsplit, const int64_t* __restrict__ Gdev,
+                               const uint64_t* __restrict__ partial, Mod M, uint64_t* __restrict__ out, int64_t ldo) {
   pdl_enter();
+  if (Gdev) gsplit = eval_tc_splits(gsplit, *Gdev);
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= T * S) return;
   int s = (int)(idx / T);
@@ -624,11 +627,19 @@ struct EvalWs {
   uint64_t *tabY, *tabZ, *tabC, *a, *htab, *U, *Wp, *UP, *UPq, *Uq, *partial;
   int64_t *start, *order, *Gdev, *total;
   int32_t *gid, *cnt, *tg, *tp;
+  EvalTcWs tc;
 };
-// fast: the probes go through the transposed tree (its own workspace), so
-// the matrix-vector kernel's tables are not carved
-static EvalWs carve_eval(Carver& cv, int64_t Tf, int nv, int k, int S, int64_t T, int gsplit, bool fast = false) {
+// The three ways to the same probes: the integer ring kernel, the tensor
+// cores, the transposed tree.
+enum EvalMethod { EVAL_RING, EVAL_TC, EVAL_TREE };
+static EvalMethod eval_method(const zr_ctx* ctx, int64_t T, int64_t Tf, int S) {
+  if (use_fast_probes(ctx, T, Tf, S)) return EVAL_TREE;
+  return use_tc_probes(T, Tf, S) ? EVAL_TC : EVAL_RING;
+}
+static EvalWs carve_eval(Carver& cv, const zr_ctx* ctx, int64_t Tf, int nv, int k, int S, int64_t T, int gsplit,
+                         EvalMethod method) {
   EvalWs w;
+  const bool fast = method == EVAL_TREE;   // the transposed tree has its own workspace
   const int64_t Tn = Tf > 0 ? Tf : 1;
   const uint64_t H = hash_slots(Tn);
   w.tabY = cv.take<uint64_t>((size_t)(k > 0 ? k : 1) * kPowTab);
@@ -643,7 +654,8 @@ static EvalWs carve_eval(Carver& cv, int64_t Tf, int nv, int k, int S, int64_t T
   w.tp = cv.take<int32_t>(Tn);
   w.start = cv.take<int64_t>(Tn);
   w.order = cv.take<int64_t>(Tn);
-  const int64_t Tr = (fast && Tn <= kFastMaxT) ? 1 : Tn;   // kept when the fast path may fall back
+  if (method == EVAL_TC) w.tc = carve_eval_tc(cv, ctx, Tn, S, T);
+  const int64_t Tr = (method == EVAL_TC || (fast && Tn <= kFastMaxT)) ? 1 : Tn;   // kept when the tree may fall back
   w.Wp = cv.take<uint64_t>((size_t)ring_words(S, Tr));
   w.UP = cv.take<uint64_t>((size_t)Tr * 32);
   w.UPq = cv.take<uint64_t>((size_t)Tr * 32);
@@ -654,16 +666,23 @@ static EvalWs carve_eval(Carver& cv, int64_t Tf, int nv, int k, int S, int64_t T
   return w;
 }
 
-// The merged weights in plain layout for the transposed tree, W[s G + g],
-// times u_g when the probes start at the first power (offset 1).
+// The merged weights in plain layout, W[s ld + g] (ld = 0: G), for the
+// transposed tree and the tensor cores, times u_g when the probes start at
+// the first power (offset 1); with Wq also the Shoup quotients.
 __global__ void __launch_bounds__(kWeightThreads)
-    k_eval_weights(int64_t G, int64_t Tf, int S, const int64_t* __restrict__ start, const int32_t* __restrict__ cnt,
+    k_eval_weights(const int64_t* __restrict__ Gdev, int64_t ld, int64_t Tf, int S, const int64_t* __restrict__ start, const int32_t* __restrict__ cnt,
                    const int64_t* __restrict__ order, const uint64_t* __restrict__ a, const uint8_t* __restrict__ exps,
                    int nv, int k, const uint64_t* __restrict__ tabC, const uint64_t* __restrict__ U, int offset, Mod M,
-                   uint64_t* __restrict__ W) {
+                   uint64_t* __restrict__ W, uint64_t* __restrict__ Wq) {
   pdl_enter();
+  const int64_t G = *Gdev;
+  if (ld == 0) ld = G;
   group_weights(G, Tf, S, S, start, cnt, order, a, exps, nv, k, tabC, M, [](int j) { return j; },
-                [&](int64_t g, int s, uint64_t r) { W[(int64_t)s * G + g] = offset ? mul_mod(r, U[g], M) : r; });
+                [&](int64_t g, int s, uint64_t r) {
+                  if (offset) r = mul_mod(r, U[g], M);
+                  W[(int64_t)s * ld + g] = r;
+                  if (Wq) Wq[(int64_t)s * ld + g] = shoup_pre(r, M);
+                });
 }
 
 // The evaluation itself, with its scratch at `base` (capacity checked by the caller).
@@ -679,9 +698,10 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   const int nv = f->nv;
   const uint64_t H = hash_slots(Tf > 0 ? Tf : 1);
   const int gsplit = eval_gsplit(ctx, T, S, Tf);
-  const bool fast = use_fast_probes(ctx, T, Tf, S);
+  const EvalMethod method = eval_method(ctx, T, Tf, S);
+  const bool fast = method == EVAL_TREE;
   Carver cv(base);
-  const EvalWs w = carve_eval(cv, Tf, nv, k, S, T, gsplit, fast);
+  const EvalWs w = carve_eval(cv, ctx, Tf, nv, k, S, T, gsplit, method);
 
   if (T <= 0) return ZR_OK;
   if (Tf == 0) {
@@ -731,13 +751,26 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
     uint64_t* W = reinterpret_cast<uint64_t*>(*fws);
     {
       const int64_t want = cdiv(G * S, 256), cap = 8ll * (ctx->sms ? ctx->sms : 152);
-      launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, G, Tf, S,
-               w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, W);
+      launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev, (int64_t)0,
+               Tf, S, w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, W, (uint64_t*)nullptr);
       note_launch();
     }
     return fast_probes_enqueue(ctx, G, w.U, W, G, S, T, out, ldo, *fws + wbytes, st);
   }
   // the group count stays on the device: the kernels read it, sized for Tf groups
+  if (method == EVAL_TC) {
+    const int64_t want = cdiv(Tn * S, 256), cap = 8ll * (ctx->sms ? ctx->sms : 152);
+    launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev,
+             eval_tc_ld(Tn), Tf, S, w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, w.tc.W, w.tc.Wq);
+    note_launch();
+    launch_eval_tc(ctx, w.tc, w.Gdev, Tn, w.U, S, T, out, ldo, status, st);
+    if (w.tc.gsplit > 1) {
+      launch_k(k_eval_combine, dim3(cdiv(T * S, 256)), dim3(256), 0, st, T, S, w.tc.gsplit, w.Gdev, w.tc.partial, M,
+               out, ldo);
+      note_launch();
+    }
+    return cuda_err(ctx, cudaGetLastError(), "zr_zippel_probes");
+  }
   const RingLayout L = ring_layout(S, Tn);
   int rw = 0;
   for (int b = 0; b < L.nb; b++) rw += L.bw[b];
@@ -753,7 +786,8 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   }
   launch_ring(T, S, offset, w.Gdev, Tn, gsplit, w.UP, w.UPq, w.U, w.Uq, w.Wp, L, M, out, ldo, w.partial, status, st);
   if (gsplit > 1) {
-    launch_k(k_eval_combine, dim3(cdiv(T * S, 256)), dim3(256), 0, st, T, S, gsplit, w.partial, M, out, ldo);
+    launch_k(k_eval_combine, dim3(cdiv(T * S, 256)), dim3(256), 0, st, T, S, gsplit, (const int64_t*)nullptr, w.partial, M,
+             out, ldo);
     note_launch();
   }
   return cuda_err(ctx, cudaGetLastError(), "zr_zippel_probes");
@@ -761,7 +795,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
 
 size_t probes_ws_need(const zr_ctx* ctx, const zr_poly* f, int k, int S, int64_t T) {
   Carver cv(nullptr);
-  carve_eval(cv, f->T, f->nv, k, S, T, eval_gsplit(ctx, T, S, f->T), use_fast_probes(ctx, T, f->T, S));
+  carve_eval(cv, ctx, f->T, f->nv, k, S, T, eval_gsplit(ctx, T, S, f->T), eval_method(ctx, T, f->T, S));
   return cv.off;
 }
 

@@ -203,6 +203,8 @@ double probe_work(const zr_ctx* ctx, int64_t T, int S, int64_t Tf);
 // falls back to the matrix-vector kernel when G > kFastMaxT
 constexpr int kFastProbeMaxS = 64;            // columns of the fast evaluator
 bool use_fast_probes(const zr_ctx* ctx, int64_t T, int64_t Tf, int S);
+// whether the matrix-vector product of the others runs on the tensor cores
+bool use_tc_probes(int64_t T, int64_t Tf, int S);
 size_t fast_probes_ws_need(int64_t G, int64_t T, int S);
 zr_status fast_probes_enqueue(zr_ctx* ctx, int64_t G, const uint64_t* U, const uint64_t* W, int64_t ldw, int S,
                               int64_t T, uint64_t* out, int64_t ldo, char* ws, cudaStream_t st);
@@ -219,6 +221,27 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
 zr_status probes_impl(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y, int S, const uint64_t* samples,
                       const uint64_t* z, int64_t T, int offset, uint64_t* out, int64_t ldo, uint32_t* status,
                       cudaStream_t st, int lane = -1);
+
+// the evaluator's product on the tensor cores (zr_eval_tc.cu): scratch for Tn
+// >= G groups (W: weights, W[s ld + g], ld = eval_tc_ld(Tn), times u_g^off;
+// Wq: their Shoup quotients)
+struct EvalTcWs {
+  uint64_t *W = nullptr, *Wq = nullptr, *giant = nullptr, *partial = nullptr;
+  unsigned char* pack = nullptr;
+  int gsplit = 1;
+};
+int64_t eval_tc_ld(int64_t Tn);
+// the splits the kernel uses for the G groups counted on the device: at least
+// eight k-steps (of 16 groups) each
+__host__ __device__ inline int eval_tc_splits(int gsplit, int64_t G) {
+  const int64_t most = (G + 127) / 128;
+  return most < 1 ? 1 : (most < gsplit ? (int)most : gsplit);
+}
+EvalTcWs carve_eval_tc(Carver& cv, const zr_ctx* ctx, int64_t Tn, int S, int64_t T);
+// out[s ldo + i] = sum_{g < *Gdev} W[g][s] U[g]^i, i < T, or the splits' partial
+// sums (gsplit > 1)
+void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t Tn, const uint64_t* U, int S, int64_t T,
+                    uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st);
 
 // argument check of a reconstruction request (zr_recon.cu)
 zr_status check_recon_args(zr_ctx* ctx, const zr_blackbox* bb, const zr_recon_params* prm);
