@@ -756,7 +756,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       const BDesc& d = SB.hD[i];
       const bool ax = fast_aux(ctx, j);
       zr_status r = fast_solve_enqueue(ctx, d.T, d.S, d.v, d.vp, d.b, d.ldb, d.part, d.denp,
-                                       SB.fast_ws + (size_t)j * P.fast_slot, ctx->fstream[j],
+                                       SB.fast_ws + (size_t)j * P.fast_slot, d.status, ctx->fstream[j],
                                        ax ? ctx->faux[j] : nullptr, ctx->faux_fork[j], ctx->faux_join[j]);
       if (r) return r;
     }
@@ -805,7 +805,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       if (!P.fast[i]) continue;
       const BDesc& d = SB.hD[i];
       const bool ax = fast_aux(ctx, 4);
-      zr_status r = fast_solve_enqueue(ctx, d.T, d.S, d.v, d.vp, d.b, d.ldb, d.part, d.denp, SB.fast_ws, st,
+      zr_status r = fast_solve_enqueue(ctx, d.T, d.S, d.v, d.vp, d.b, d.ldb, d.part, d.denp, SB.fast_ws, d.status, st,
                                        ax ? ctx->faux[4] : nullptr, ctx->faux_fork[4], ctx->faux_join[4]);
       if (r) return r;
     }

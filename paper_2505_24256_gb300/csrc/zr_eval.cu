@@ -75,38 +75,57 @@ __global__ void k_eval_init(const uint64_t* __restrict__ y, int k, const uint64_
 // per term: its anchor value u_t, its weight without the new variable,
 // a_t = coef_t prod_{m>k} z_m^{e_{t,m}}, and its hash slot; the thread that
 // fills a slot numbers the group
-__global__ void k_eval_terms(int64_t Tf, int nv, const uint8_t* __restrict__ exps, const uint64_t* __restrict__ coef,
+__global__ void __launch_bounds__(256) k_eval_terms(int64_t Tf, int nv, const uint8_t* __restrict__ exps, const uint64_t* __restrict__ coef,
                              int k, const uint64_t* __restrict__ tabY, const uint64_t* __restrict__ tabZ, Mod M,
                              uint64_t* __restrict__ a, uint64_t* htab, uint64_t hmask, int32_t* __restrict__ gid,
                              uint64_t* __restrict__ U, int64_t* Gdev, uint32_t* __restrict__ slot, uint32_t* status) {
   pdl_enter();
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= Tf) return;
-  const uint8_t* e = exps + t * nv;
-  uint64_t uu = 1;
-  for (int m = 0; m < k; m++) uu = mul_mod(uu, tabY[m * kPowTab + e[m]], M);
-  uint64_t c = coef[t];
-  if (c >= M.p) c -= M.p;
-  for (int m = k + 1; m < nv; m++) c = mul_mod(c, tabZ[m * kPowTab + e[m]], M);
-  a[t] = c;
-  // insert the key; equal keys share a slot
-  uint64_t idx = ehash(uu) & hmask;
-  for (uint64_t probe = 0; probe <= hmask; probe++) {
-    unsigned long long prev = atomicCAS((unsigned long long*)&htab[idx], (unsigned long long)kEmpty,
-                                        (unsigned long long)uu);
-    if (prev == kEmpty) {
-      const int32_t g = (int32_t)atomicAdd((unsigned long long*)Gdev, 1ull);
-      gid[idx] = g;
-      U[g] = uu;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint64_t uu = 1, found = ~0ull;
+  bool won = false;
+  if (t < Tf) {
+    const uint8_t* e = exps + t * nv;
+    for (int m = 0; m < k; m++) uu = mul_mod(uu, tabY[m * kPowTab + e[m]], M);
+    uint64_t c = coef[t];
+    if (c >= M.p) c -= M.p;
+    for (int m = k + 1; m < nv; m++) c = mul_mod(c, tabZ[m * kPowTab + e[m]], M);
+    a[t] = c;
+    // insert the key; equal keys share a slot
+    uint64_t idx = ehash(uu) & hmask;
+    for (uint64_t probe = 0; probe <= hmask; probe++) {
+      unsigned long long prev = atomicCAS((unsigned long long*)&htab[idx], (unsigned long long)kEmpty,
+                                          (unsigned long long)uu);
+      won = prev == kEmpty;
+      if (won || prev == uu) {
+        found = idx;
+        break;
+      }
+      idx = (idx + 1) & hmask;
     }
-    if (prev == kEmpty || prev == uu) {
-      slot[t] = (uint32_t)idx;
-      return;
-    }
-    idx = (idx + 1) & hmask;
+    slot[t] = (uint32_t)found;
+    if (found == ~0ull) atomicOr(status, ST_HASH_FULL);
   }
-  slot[t] = ~0u;
-  atomicOr(status, ST_HASH_FULL);
+  // a block's new groups take their numbers with one addition (one per warp
+  // took 0.6 ms for the 2^20 groups of 9.4 million terms)
+  __shared__ int warp_new[8];
+  __shared__ unsigned long long first;
+  const unsigned winners = __ballot_sync(0xffffffffu, won);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) warp_new[warp] = __popc(winners);
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < 8; w++) {
+    if (w < warp) before += warp_new[w];
+    total += warp_new[w];
+  }
+  if (threadIdx.x == 0 && total) first = atomicAdd((unsigned long long*)Gdev, (unsigned long long)total);
+  __syncthreads();
+  if (won) {
+    const int32_t g = (int32_t)(first + before + __popc(winners & ((1u << lane) - 1)));
+    gid[found] = g;
+    U[g] = uu;
+  }
 }
 
 // tg[t] = the term's group (over its hash slot), tp[t] = its place in the
@@ -153,19 +172,23 @@ __global__ void k_eval_scatter(int64_t Tf, const int32_t* __restrict__ tg, const
 // s < S <= 256, handed to store(g, j, value) for the row entries j < rw,
 // column(j) the entry's column s (negative: padding, zero).
 //
-// Short groups: a thread per entry.  Long ones (eight terms and more on
-// average, the early variables of a reconstruction): a block per group, its
-// terms staged 256 at a time, a warp every eighth of them, lanes the columns;
+// Many or short groups: a thread per entry.  Few long ones (eight terms and
+// more on average and at most kWeightEntries entries, or 64 terms and more:
+// the early variables of a reconstruction): a block per group, its terms
+// staged 256 at a time, a warp every eighth of them, lanes the columns;
 // a thread per entry then ran through hundreds of dependent gathers (0.043 ms
 // a call on average over a reconstruction of 8000 terms against 0.012 ms).
+// With entries enough to fill the GPU it is the other way round: 0.34 against
+// 3.9 ms for 2^20 groups of nine terms.
 constexpr int kWeightThreads = 256;
+constexpr int64_t kWeightEntries = 1 << 16;
 template <class Column, class Store>
 __device__ __forceinline__ void group_weights(int64_t G, int64_t Tf, int S, int rw, const int64_t* __restrict__ start,
                                               const int32_t* __restrict__ cnt, const int64_t* __restrict__ order,
                                               const uint64_t* __restrict__ a, const uint8_t* __restrict__ exps, int nv,
                                               int k, const uint64_t* __restrict__ tabC, const Mod& M, Column column,
                                               Store store) {
-  if (G * 8 <= Tf) {
+  if ((G * 8 <= Tf && G * rw <= kWeightEntries) || G * 64 <= Tf) {
     __shared__ uint64_t sa[kWeightThreads], vals[256], red[kWeightThreads / 32][32];
     __shared__ uint8_t se[kWeightThreads];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -711,7 +734,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   const int64_t Tn = Tf;
   const int nz = z && nv > k + 1 ? nv : 0;
   {
-    const int64_t cap = 2ll * (ctx->sms ? ctx->sms : 152);
+    const int64_t cap = 8ll * (ctx->sms ? ctx->sms : 152);
     const unsigned fill = (unsigned)std::min<int64_t>(cdiv((int64_t)H, kPowTab), cap);
     launch_k(k_eval_init, dim3(k + nz + S + fill), dim3(kPowTab), 0, st, y, k, z, nz, samples, S, M, w.tabY, w.tabZ,
              w.tabC, w.htab, H, w.cnt, Tn, w.Gdev, w.total);

@@ -342,12 +342,7 @@ void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t
   const Mod& M = ctx->M;
   const int64_t ld = eval_tc_ld(Tn);
   const int A = etc_a(T);
-  auto pow2 = [&](int e) {
-    unsigned __int128 r = 1;
-    for (int i = 0; i < e; i++) r = r * 2 % M.p;
-    return (uint64_t)r;
-  };
-  const TcMod K = {pow2(96), (uint64_t)(((unsigned __int128)pow2(110) + pow2(154)) % M.p)};
+  const TcMod K = tc_mod(M);
   launch_k(k_etc_pack, dim3((unsigned)(ld / 8)), dim3(kTcRows), 0, st, U, Gdev, A, ld, M, (uint4*)w.pack, w.giant);
   const int tiles = (int)cdiv((int64_t)A * S, kEtcNC), sms = ctx->sms ? ctx->sms : 152;
   launch_k(k_eval_tc, dim3((unsigned)std::min(tiles * w.gsplit, sms)), dim3(kEtcThreads), kEtcSmem, st, T, S, Gdev, A,

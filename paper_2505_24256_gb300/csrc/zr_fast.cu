@@ -16,10 +16,11 @@
 //            truncated to deg L terms: X_L[m] = sum_{i <= deg R} r_i X_P[m+i],
 //            a middle product computed as a cyclic convolution of size 2^l of
 //            the reversed X_P with R, read backwards; likewise for R.
-//   leaves   at a block P of 128 roots, X_P is the expansion of a
+//   leaves   at a block P of 128 or 256 roots, X_P is the expansion of a
 //            generating function whose numerator is N(v_j) / (M/P)(v_j) at
 //            the block's roots; <q^P_j, X_P> with q^P_j = P / (z - v_j) gives
-//            N(v_j) directly (the quadratic method on 128 roots).
+//            N(v_j) directly (the quadratic method on the block, its products
+//            on the tensor cores: zr_fast_leaf.cu).
 //   denominators   M'(v_j) is the same evaluation with N = M', whose
 //            expansion M'/M = sum_k (sum_j v_j^k) z^(-k-1) holds the power
 //            sums of the nodes: summed directly (T^2 Shoup steps beside the
@@ -978,6 +979,7 @@ constexpr int kNewtonClusterLog = 14;
 // Tree level l <= kFusedLog: the children of node P as full monic
 // polynomials (modulo prime `me`) -> spectra (kept in spec for the descent)
 // -> product -> inverse -> coefficients of P (the wrapped z^n taken off).
+// spec null: the descent does not come here.
 __global__ void __launch_bounds__(kClusterThreadsMax) k_tree_cluster(const uint64_t* __restrict__ below, int64_t T,
                                                                 int64_t Tp, int logn, NttConsts C, CrtScale sc, Mod M,
                                                                 const uint2* __restrict__ tw, int logN,
@@ -999,11 +1001,13 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_tree_cluster(const uint6
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);
-  uint32_t* sp = spec + (int64_t)me * 2 * Tp + (2 * P << logn);
+  uint32_t* sp = spec ? spec + (int64_t)me * 2 * Tp + (2 * P << logn) : nullptr;
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const uint32_t x = fsm[sw(k)], y = fsm[sw(n + k)];
-    sp[k] = x;
-    sp[n + k] = y;
+    if (sp) {
+      sp[k] = x;
+      sp[n + k] = y;
+    }
     fsm[sw(k)] = mont32(sub_if(x, 2 * q), sub_if(y, 2 * q), q, qi);
   }
   if (coef == nullptr) return;                   // the children's spectra only (every CTA alike)
@@ -1122,56 +1126,12 @@ __global__ void __launch_bounds__(kLeaf) k_fast_leafpoly(const uint64_t* __restr
   if (t < cnt) coef[base + t] = buf[cur][t];
 }
 
-// Leaf values: for root j of block P (degree d), val_r = <q^P_j, X_P^(r)>,
-// q^P_{j,d-1} = 1, q^P_{j,k-1} = p_k + v_j q^P_{j,k}.  Rows r < R - 1 are the
-// right-hand sides (written to part[r ldp + j]), row R - 1 the power sums
-// (M'(v_j), written to den[j]).  A CTA takes one block and one group of
-// kLeafCols rows (blockIdx.y), each thread one root, rerunning the chain per
-// group so that the groups run in parallel.
-constexpr int kLeafCols = 4;
-
-__global__ void __launch_bounds__(kLeaf) k_fast_leafval(const uint64_t* __restrict__ coef7,
-                                                        const uint64_t* __restrict__ X, int R, int64_t T, int64_t Tp,
-                                                        const uint64_t* __restrict__ v, const uint64_t* __restrict__ vp,
-                                                        Mod M, uint64_t* __restrict__ part, int64_t ldp,
-                                                        uint64_t* __restrict__ den) {
-  pdl_enter();
-  __shared__ uint64_t pc[kLeaf];                 // block polynomial
-  __shared__ uint64_t xs[kLeafCols][kLeaf];      // this group's X rows
-  const int64_t base = (int64_t)blockIdx.x * kLeaf;
-  const int r0 = blockIdx.y * kLeafCols;
-  const int d = (int)((T - base) < kLeaf ? (T - base) : kLeaf);
-  const int t = threadIdx.x;
-  if (t < d) pc[t] = coef7[base + t];
-#pragma unroll
-  for (int c = 0; c < kLeafCols; c++)
-    if (t < d && r0 + c < R) xs[c][t] = X[(int64_t)(r0 + c) * Tp + base + t];
-  __syncthreads();
-  if (t >= d) return;
-  const int64_t j = base + t;
-  const uint64_t vj = v[j], vpj = vp[j];
-  Acc8 acc[kLeafCols];
-#pragma unroll
-  for (int c = 0; c < kLeafCols; c++) acc[c] = Acc8{0, 0, 0, 0, 0, 0, 0, 0};
-  uint64_t q = 1;
-  for (int k = d - 1; k >= 0; k--) {
-    const uint64_t qc = canon(q, M);
-    const uint32_t x0 = lo32(qc), x1 = hi32(qc);
-#pragma unroll
-    for (int c = 0; c < kLeafCols; c++)
-      if (r0 + c < R) {
-        const uint64_t w = xs[c][k];
-        mac8(acc[c], x0, x1, lo32(w), hi32(w));
-      }
-    q = canon(shoup_lazy(qc, vj, vpj, M), M) + pc[k];
-  }
-#pragma unroll
-  for (int c = 0; c < kLeafCols; c++) {
-    const int r = r0 + c;
-    if (r < R - 1) part[(int64_t)r * ldp + j] = acc8_value(acc[c], M);
-    else if (r == R - 1) den[j] = acc8_value(acc[c], M);
-  }
-}
+// The descent stops at blocks of 2^7 roots, of 2^8 from kDescLeaf8T unknowns on,
+// whose values launch_leaf_tc takes.  Measured on GB300 (whole step, leaves of
+// 2^7 / 2^8 / 2^9): T = 1024, S = 21: 0.207 / 0.208 / 0.220 ms; 3000, 21: 0.296
+// / 0.293 / 0.300; 10^4, 21: 0.566 / 0.554 / 0.561; 125000, 9: 2.92 / 2.81 /
+// 2.80; 2^20, 9: 23.5 / 22.3 / 22.3.
+constexpr int64_t kDescLeaf8T = 2048;
 
 // X0[r][k] = b[r ldb + k] (r < S), X0[S][k] = power sums (k < T), rows r0 .. r0 + nr - 1
 __global__ void k_stage_rhs(const uint64_t* __restrict__ b, int64_t ldb, int S, const uint64_t* __restrict__ ps,
@@ -1710,9 +1670,10 @@ struct FastRun {
   // 128 2^Lt words each) and the children's spectra spec[l - 1] (kNP 2T'
   // words each); Z: kNP T' words of scratch.  Without `root` the top level
   // may stop at its children's spectra (coef[Lt], M itself, left unwritten
-  // when that level runs on a cluster).
+  // when that level runs on a cluster).  The spectra of levels l <= lspec may
+  // be left unwritten.
   void tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::vector<uint64_t*>& coef,
-            const std::vector<uint32_t*>& spec, uint32_t* Z, bool root = true);
+            const std::vector<uint32_t*>& spec, uint32_t* Z, bool root = true, int lspec = 0);
   // g = 1 / f mod z^prec (f_0 = 1, nf coefficients): Newton's iteration, the
   // first steps in one CTA; g holds 2 prec words, e prec words, A, B, Z
   // kNP 2^ceil(log2(2 prec)) words each
@@ -1824,7 +1785,7 @@ void configure_fused() {
 }
 
 void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::vector<uint64_t*>& coef,
-                   const std::vector<uint32_t*>& spec, uint32_t* Z, bool root) {
+                   const std::vector<uint32_t*>& spec, uint32_t* Z, bool root, int lspec) {
   const int logT = kLeafLog + Lt;
   launch_k(k_fast_leafpoly, cdivu(T, kLeaf), kLeaf, 0, st, v, T, M, coef[0]);
   note_launch();
@@ -1834,7 +1795,8 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
     const int64_t nodes = (T + (1ll << logn) - 1) >> logn;
     if (cluster_level(ctx, logn, nodes)) {
       const cudaError_t e = launch_cluster(k_tree_cluster, nodes, cluster_threads(logn), sizeof(uint32_t) * 2 << logn,
-                                           st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M, tw, logN, sp,
+                                           st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M, tw, logN,
+                                           l <= lspec ? (uint32_t*)nullptr : sp,
                                            (l == Lt && !root) ? (uint64_t*)nullptr : coef[l]);
       if (e == cudaSuccess) continue;
       (void)cudaGetLastError();
@@ -2010,13 +1972,14 @@ zr_status fast_tables_for(zr_ctx* ctx, int64_t T, cudaStream_t st) {
 // are on the device already; ws holds fast_ws_need(T, S + 1) bytes.
 zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, const uint64_t* vp,
                              const uint64_t* b, int64_t ldb, uint64_t* part, uint64_t* den, char* ws,
-                             cudaStream_t st, cudaStream_t aux, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
+                             uint32_t* status, cudaStream_t st, cudaStream_t aux, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
   const int R = S + 1;
   Carver cv(ws);
   FastWs w = carve_fast(cv, T, R);
   const int64_t Tp = w.Tp;
   const int Lt = w.Lt;
   const int logT = kLeafLog + Lt;
+  const int l0 = T >= kDescLeaf8T ? 1 : 0;   // the descent stops at level 7 + l0 (l0 <= Lt)
   zr_status r = ensure_ntt_tables(ctx, logT + 1, st);
   if (r) return r;
   const NttConsts& C = ctx->ntt;
@@ -2054,10 +2017,11 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
     prof_add(ctx, PH_PSUM, pa, pb, (double)T * (double)T);
     launch_k(k_power_sums_add, cdivu(T, 256), 256, 0, st, (const uint64_t*)w.psp, T, ps.nb, M, w.ps);
     note_launches(3);
-    Fa.tree(v, T, Tp, Lt, w.coef, w.spec, w.Z, false);   // M itself is not needed: the descent takes its children
+    // M itself is not needed unless it is the only leaf: the descent takes its children
+    Fa.tree(v, T, Tp, Lt, w.coef, w.spec, w.Z, l0 == Lt, l0);
     if (fork) cudaEventRecord(ev_join, sa);
   } else {
-    F.tree(v, T, Tp, Lt, w.coef, w.spec, w.Z);
+    F.tree(v, T, Tp, Lt, w.coef, w.spec, w.Z, true, l0);
   }
   const uint64_t* m = w.coef[Lt];   // M without its leading 1 (written on the Newton path only)
   // descent from the root (node size T') to the leaf blocks of nr rows from
@@ -2067,7 +2031,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
     uint64_t* Xn = w.X1 + (size_t)r0 * Tp;
     uint32_t* XH = w.XH + (size_t)r0 * kNP * Tp;
     uint32_t* Y = w.Y + (size_t)2 * r0 * kNP * Tp;
-    for (int l = Lt; l >= 1; l--) {
+    for (int l = Lt; l > l0; l--) {
       const int logn = kLeafLog + l;
       const int64_t nodes = (T + (1ll << logn) - 1) >> logn;
       bool done = false;
@@ -2141,11 +2105,8 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       cudaStreamWaitEvent(st, ev_join, 0);
     }
   }
-  uint64_t* X = (Lt & 1) ? w.X1 : w.X0;     // where Lt swaps leave the rows
-  // leaves
-  launch_k(k_fast_leafval, dim3(cdivu(T, kLeaf), (unsigned)((R + kLeafCols - 1) / kLeafCols)), kLeaf, 0, st, 
-      w.coef[0], X, R, T, Tp, v, vp, M, part, T, den);
-  note_launch();
+  uint64_t* X = ((Lt - l0) & 1) ? w.X1 : w.X0;   // where the levels' swaps leave the rows
+  launch_leaf_tc(w.coef[l0], X, R, kLeafLog + l0, T, Tp, v, vp, M, part, T, den, status, st);
   return cuda_err(ctx, cudaGetLastError(), "fast solve");
 }
 

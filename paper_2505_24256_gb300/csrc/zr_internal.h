@@ -187,8 +187,12 @@ size_t fast_ws_need(int64_t T, int R);
 // (aux, ev_fork, ev_join: a second stream and two events on which the power
 // sums run beside the right-hand sides' descent; null: all on st)
 zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, const uint64_t* vp, const uint64_t* b,
-                             int64_t ldb, uint64_t* part, uint64_t* den, char* ws, cudaStream_t st,
+                             int64_t ldb, uint64_t* part, uint64_t* den, char* ws, uint32_t* status, cudaStream_t st,
                              cudaStream_t aux = nullptr, cudaEvent_t ev_fork = nullptr, cudaEvent_t ev_join = nullptr);
+// the leaves of the fast solve (zr_fast_leaf.cu)
+void launch_leaf_tc(const uint64_t* coef, const uint64_t* X, int R, int ll, int64_t T, int64_t Tp, const uint64_t* v,
+                    const uint64_t* vp, const Mod& M, uint64_t* part, int64_t ldp, uint64_t* den, uint32_t* status,
+                    cudaStream_t st);
 // whether a system of T unknowns takes the fast path in this context
 // (batch_n: the number of systems in the call; alone, the fast path is taken from a smaller T)
 bool use_fast_solve(const zr_ctx* ctx, int64_t T, int S, int batch_n = 1);

@@ -1,7 +1,8 @@
 // zr_tc.cuh -- exact products of 63-bit residues on the tensor cores.
 //
 // A residue x, taken centred (|x| <= p / 2 < 2^62), is written in eight
-// balanced base-256 digits, x = sum_i d_i 256^i with -128 <= d_i <= 127; every
+// balanced base-256 digits, x = sum_i d_i 256^i with -128 <= d_i <= 127 (or
+// any 64-bit word y as y - 0x8080..80, the constant corrected later); every
 // digit is exact in bf16 (eight significand bits).  A sum over k <= 128 of
 // products x_k y_k has the antidiagonal sums
 //     D_m = sum_k sum_{i+j=m} d_i(x_k) d_j(y_k),   m = 0 .. 14,
@@ -33,25 +34,18 @@ constexpr int kTcDiags = 2 * kTcLimbs - 1;
 constexpr int kTcRows = 128;        // rows of a tile: the tensor memory's lanes
 constexpr int kTcChunk = 128;       // k summed in the tensor memory at a time (the bound above)
 
-// Digits of eight residues (consecutive k of one row): out[i] holds digit i of
-// all eight as bf16.  Adding 128 to every digit turns them into the bytes of
-// x + 0x8080..80; a byte b becomes b - 128 through the bf16 numbers 128 + (b &
-// 127) and 128 or 256 (ulp 1 in [128, 256)).
-__device__ __forceinline__ void tc_digits(const uint64_t (&x)[8], uint64_t p, uint4 (&out)[kTcLimbs]) {
-  const uint64_t half = p >> 1;
-  uint32_t lo[8], hi[8];
-#pragma unroll
-  for (int k = 0; k < 8; k++) {
-    const uint64_t y = (x[k] > half ? x[k] - p : x[k]) + 0x8080808080808080ull;
-    lo[k] = lo32(y);
-    hi[k] = hi32(y);
-  }
+// Digits of eight words y (consecutive k of one row): out[i] holds byte i less
+// 128 of all eight as bf16, the digits of y - 0x8080..80.  A byte b becomes b -
+// 128 through the bf16 numbers 128 + (b & 127) and 128 or 256 (ulp 1 in [128,
+// 256)).
+constexpr uint64_t kTcBias = 0x8080808080808080ull;
+__device__ __forceinline__ void tc_bytes(const uint64_t (&y)[8], uint4 (&out)[kTcLimbs]) {
 #pragma unroll
   for (int i = 0; i < kTcLimbs; i++) {
     uint32_t w[4];
 #pragma unroll
     for (int q = 0; q < 4; q++) {
-      const uint32_t a = i < 4 ? lo[2 * q] : hi[2 * q], b = i < 4 ? lo[2 * q + 1] : hi[2 * q + 1];
+      const uint32_t a = i < 4 ? lo32(y[2 * q]) : hi32(y[2 * q]), b = i < 4 ? lo32(y[2 * q + 1]) : hi32(y[2 * q + 1]);
       const uint32_t two = __byte_perm(a, b, 0x4400u + 0x1111u * (i & 3));   // bytes i, i of a; i, i of b
       const uint32_t u = (two & 0x007f007fu) | 0x43004300u, v = (~two & 0x00800080u) | 0x43004300u;
       __nv_bfloat162 du, dv;
@@ -62,6 +56,14 @@ __device__ __forceinline__ void tc_digits(const uint64_t (&x)[8], uint64_t p, ui
     }
     out[i] = make_uint4(w[0], w[1], w[2], w[3]);
   }
+}
+// Digits of eight residues, centred: at most 65 in magnitude for the top one.
+__device__ __forceinline__ void tc_digits(const uint64_t (&x)[8], uint64_t p, uint4 (&out)[kTcLimbs]) {
+  const uint64_t half = p >> 1;
+  uint64_t y[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) y[k] = (x[k] > half ? x[k] - p : x[k]) + kTcBias;
+  tc_bytes(y, out);
 }
 
 // ---- tcgen05 ---------------------------------------------------------------------
@@ -156,10 +158,10 @@ __device__ __forceinline__ void tc_carry(TcAcc& a) {
 // The chunk sums D_0 .. D_14 of four columns (addr + m NC + c) added into acc.
 //
 // Sum by sum the excess over a balanced digit is carried on, D_m = 256 q + r,
-// q = round(D_m / 256) added to D_{m+1}, all exact: the centred top digits
-// are at most 65 in magnitude, so |D_m| <= 128 (6 * 2^14 + 2 * 128 * 65) <
-// 2^24 - 2^17 leaves room for the carry, and q + 3 * 2^22 rounds to an
-// integer.  Three digits make a 24-bit word, one conversion to integer each:
+// q = round(D_m / 256) added to D_{m+1}, all exact: one operand at least is
+// centred, its top digits at most 65 in magnitude, so |D_m| <= 128 (7 * 2^14 +
+// 128 * 65) < 2^24 - 2^17 leaves room for the carry, and q + 3 * 2^22 rounds
+// to an integer.  Three digits make a 24-bit word, one conversion to integer each:
 // conversions run at 16 lanes per SM and clock, and fifteen of them with
 // 64-bit additions took 4430 clocks per 128 x 32 outputs, this 3300.
 template <int NC>
@@ -191,6 +193,7 @@ __device__ __forceinline__ void tc_add_chunk(uint32_t addr, TcAcc* acc) {
 struct TcMod {
   uint64_t c96, bias;
 };
+TcMod tc_mod(const Mod& M);   // host
 __device__ __forceinline__ uint64_t tc_value(TcAcc a, const TcMod& K, const Mod& M) {
   tc_carry(a);
   const int64_t x0 = (int64_t)a.w[0] + ((int64_t)a.w[1] << 24), x1 = (int64_t)a.w[2] + ((int64_t)a.w[3] << 24),

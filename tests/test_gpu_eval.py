@@ -93,3 +93,7 @@ def test_probes_tensor_cores_long_sums(ctx, orc):
     sidx, iidx = st.below(40, S).astype(np.int64), st.below(40, T).astype(np.int64)
     want = orc.zippel_probes_sampled(exps, coef, k, y, cs, z, sidx, iidx)
     assert np.array_equal(h64(out)[sidx, iidx], want)
+
+
+def test_probes_many_groups_of_several_terms(ctx, orc):
+    test_probes_groups(ctx, orc, 90000, 5, 4, 9, 8, 31, 1)
