@@ -103,12 +103,15 @@ __global__ void k_ntt_tables(int logN, NttConsts C, uint2* __restrict__ tw, uint
 
 // Shared-memory layout of the transform kernels: logical word x lives at
 // sw(x), its bank bits XORed with bits of its 32-word row (a permutation
-// within each row).  The register passes below touch words at strides 1, 8
-// and multiples of 32; with this swizzle each of those warp accesses, and
-// every run of 32 consecutive row-aligned words, hits 32 distinct banks.
-__device__ __forceinline__ int sw(int x) { return x ^ (((x >> 5) & 7) | ((x >> 3) & 24)); }
+// within each row).  The register passes below touch 16 words at stride 1 or
+// 16, or 8 words at strides 1, 8, 16 or multiples of 32: a warp's accesses
+// then vary five bits of x (4..8; 0..3 and 8; 3..7; 0..2, 6 and 7; 0..3 and 7;
+// 0..4), and with this swizzle each of them, and every run of 32 consecutive
+// row-aligned words, hits 32 distinct banks (the five bank bits are independent
+// sums of the five).  It is linear over GF(2): sw(x ^ y) = sw(x) ^ sw(y).
+__host__ __device__ constexpr int sw(int x) { return x ^ ((x >> 5) & 15) ^ ((x >> 3) & 24) ^ ((x >> 4) & 16); }
 
-// One pass of R <= 3 butterfly stages over groups of 2^R words held in
+// One pass of R <= 4 butterfly stages over groups of 2^R words held in
 // registers (a radix-2^R pass).  Forward (Cooley-Tukey) stages s .. s+R-1:
 // a group is the words a + i 2^u (u = lt - R + 1, lt = logn - 1 - s) of one
 // block of 2^(lt+1); stage s+j pairs words 2^(R-1-j) apart with the twiddle
@@ -119,17 +122,29 @@ __device__ __forceinline__ int sw(int x) { return x ^ (((x >> 5) & 7) | ((x >> 3
 // transform position (boff + x) mod 2^logn; prime_of(x) gives its prime.
 // COLS: the buffer holds 2^cwl columns side by side instead (word x of
 // column c at x 2^cwl + c, no swizzle), one transform each; consecutive
-// threads take consecutive columns.
-template <bool INV, int R, bool COLS, class PrimeOf>
+// threads take consecutive columns.  U: the stride's logarithm when it is
+// known (the word offsets are then constants), else -1.
+//
+// The passes are bound by instruction issue: 7 per butterfly, the rest is
+// addresses, twiddle loads and shared-memory accesses, which a group of 16
+// spreads over 32 butterflies.  (13 stages as 1 + 3 + 3 + 3 + 3 took 19.5
+// instructions per butterfly, as 3 + 3 + 3 + 4 it
+// takes 16: 36 to 32 us for 720 tiles of 8192 words.)
+template <bool INV, int R, int U, bool COLS, class PrimeOf>
 __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int logn, int s, uint32_t boff,
                                            const uint2* __restrict__ tw, int logN, const NttConsts& C,
                                            PrimeOf prime_of, int cwl) {
   constexpr int NR = 1 << R;
   const int lt = logn - 1 - s;
-  const int u = INV ? lt : lt - R + 1;           // log2 of the stride within a group
-  const int blog = INV ? lt + R : lt + 1;        // log2 of the group's block
+  const int u = U >= 0 ? U : (INV ? lt : lt - R + 1);   // log2 of the stride within a group
+  const int blog = u + R;                               // log2 of the group's block
   const uint32_t pmask = (1u << logn) - 1;
   const uint32_t m = 1u << s;
+  // word i of a group sits at sw(off + a + (i << u)) = sw(off + a) ^ sw(i << u)
+  // (disjoint bits)
+  int cst[NR];
+#pragma unroll
+  for (int i = 0; i < NR; i++) cst[i] = COLS ? i << (u + cwl) : sw(i << u);
   for (int g0 = threadIdx.x; g0 < (len >> R); g0 += blockDim.x) {
     const int col = COLS ? (g0 & ((1 << cwl) - 1)) : 0;
     const int g = COLS ? (g0 >> cwl) : g0;
@@ -138,87 +153,80 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
     const uint32_t q = C.q[prime];
     const uint32_t kb = ((boff + (uint32_t)a) & pmask) >> blog;
     const uint2* __restrict__ twp = tw + ((int64_t)prime << logN);
-    uint2 w[NR - 1];
-    int wo = 0;
-#pragma unroll
-    for (int j = 0; j < R; j++) {
-      const int cnt = INV ? (1 << (R - 1 - j)) : (1 << j);
-      const uint32_t base = INV ? (m >> j) + (kb << (R - 1 - j)) : (m << j) + (kb << j);
-      // a stage's twiddles are contiguous and start at a multiple of their
-      // count: pairs load as 16 bytes
-      if (cnt == 1) {
-        w[wo] = __ldg(&twp[base]);
-      } else {
-#pragma unroll
-        for (int c = 0; c < cnt; c += 2) {
-          const uint4 t2 = __ldg(reinterpret_cast<const uint4*>(twp + base + c));
-          w[wo + c] = make_uint2(t2.x, t2.y);
-          w[wo + c + 1] = make_uint2(t2.z, t2.w);
-        }
-      }
-      wo += cnt;
-    }
-    // word addresses: for stride 1 the group lies in one row (sw(base) ^ i),
-    // for strides of 256 and more the row bits of the swizzle are the
-    // base's (sw(base) + (i << u)); strides 8 and 64 swizzle each word
-    int at[NR];
-    const int sb = sw(off + a);
-#pragma unroll
-    for (int i = 0; i < NR; i++)
-      at[i] = COLS ? (((a + (i << u)) << cwl) + col)
-                   : (u == 0 ? (sb ^ i) : (u >= 8 ? sb + (i << u) : sw(off + a + (i << u))));
+    const int sb = COLS ? (a << cwl) + col : sw(off + a);
     uint32_t x[NR];
 #pragma unroll
-    for (int i = 0; i < NR; i++) x[i] = sm[at[i]];
-    wo = 0;
+    for (int i = 0; i < NR; i++) x[i] = sm[COLS ? sb + cst[i] : sb ^ cst[i]];
 #pragma unroll
     for (int j = 0; j < R; j++) {
+      // a stage's twiddles are contiguous and start at a multiple of their
+      // count: pairs load as 16 bytes
+      constexpr int kMost = NR / 2;
+      const int cnt = INV ? (1 << (R - 1 - j)) : (1 << j);
+      const uint2* __restrict__ tj = twp + (INV ? (m >> j) + (kb << (R - 1 - j)) : (m << j) + (kb << j));
+      uint2 w[kMost];
+      if (cnt == 1) {
+        w[0] = __ldg(tj);
+      } else {
+#pragma unroll
+        for (int c = 0; c < kMost; c += 2)
+          if (c < cnt) {
+            const uint4 t2 = __ldg(reinterpret_cast<const uint4*>(tj + c));
+            w[c] = make_uint2(t2.x, t2.y);
+            w[c + 1] = make_uint2(t2.z, t2.w);
+          }
+      }
       const int hs = INV ? (1 << j) : (1 << (R - 1 - j));
 #pragma unroll
       for (int i = 0; i < NR; i++)
-        if (!(i & hs)) butterfly<INV>(x[i], x[i + hs], w[wo + (INV ? (i >> (j + 1)) : (i >> (R - j)))], q);
-      wo += INV ? (1 << (R - 1 - j)) : (1 << j);
+        if (!(i & hs)) butterfly<INV>(x[i], x[i + hs], w[INV ? (i >> (j + 1)) : (i >> (R - j))], q);
     }
 #pragma unroll
-    for (int i = 0; i < NR; i++) sm[at[i]] = x[i];
+    for (int i = 0; i < NR; i++) sm[COLS ? sb + cst[i] : sb ^ cst[i]] = x[i];
   }
 }
 
 // Stages s_lo .. logn-1 of the transforms in sm (logical words off ..
-// off + len), forward in increasing or inverse in decreasing stage order:
-// radix-8 passes, the leftover one or two stages as one pass on the
-// largest strides.  Callers synchronise before; the last pass is followed
-// by a barrier.
+// off + len), forward in increasing or inverse in decreasing stage order, in
+// ceil(K / 4) passes of three or four stages (K = logn - s_lo; one or two
+// stages when K < 3, 2 + 3 when K = 5), those of four on the smallest strides.
+// Callers synchronise before; the last pass is followed by a barrier.
 template <bool INV, bool COLS = false, class PrimeOf>
 __device__ __forceinline__ void smem_stages(uint32_t* sm, int off, int len, int logn, int s_lo, uint32_t boff,
                                             const uint2* __restrict__ tw, int logN, const NttConsts& C,
                                             PrimeOf prime_of, int cwl = 0) {
-  const int rem = (logn - s_lo) % 3;
+  const int K = logn - s_lo, np = (K + 3) >> 2;
+  const int fours = K - 3 * np;                      // passes of four; negative: that many stages fewer in the widest
+  auto pass = [&](int R, int s) {
+    const int u = INV ? logn - 1 - s : logn - s - R;
+    if (R == 4) {
+      if (COLS) radix_pass<INV, 4, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      else if (u == 0) radix_pass<INV, 4, 0, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      else if (u == 4) radix_pass<INV, 4, 4, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      else radix_pass<INV, 4, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+    } else if (R == 3) {
+      radix_pass<INV, 3, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+    } else if (R == 2) {
+      radix_pass<INV, 2, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+    } else {
+      radix_pass<INV, 1, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+    }
+    __syncthreads();
+  };
+  if (K <= 0) return;
   if (!INV) {
     int s = s_lo;
-    if (rem == 1) {
-      radix_pass<false, 1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
-    } else if (rem == 2) {
-      radix_pass<false, 2, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
-    }
-    for (s += rem; s < logn; s += 3) {
-      radix_pass<false, 3, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
+    for (int i = 0; i < np; i++) {
+      const int R = fours < 0 ? (i == 0 ? 3 + fours : 3) : (i >= np - fours ? 4 : 3);
+      pass(R, s);
+      s += R;
     }
   } else {
     int s = logn - 1;
-    for (; s - 2 >= s_lo; s -= 3) {
-      radix_pass<true, 3, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
-    }
-    if (rem == 2) {
-      radix_pass<true, 2, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
-    } else if (rem == 1) {
-      radix_pass<true, 1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      __syncthreads();
+    for (int i = np - 1; i >= 0; i--) {
+      const int R = fours < 0 ? (i == 0 ? 3 + fours : 3) : (i >= np - fours ? 4 : 3);
+      pass(R, s);
+      s -= R;
     }
   }
 }
@@ -239,10 +247,11 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
     const uint4* src = reinterpret_cast<const uint4*>(data + base);
     for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads) {
       const uint4 v = src[e];
-      sm[sw(4 * e)] = v.x;
-      sm[sw(4 * e + 1)] = v.y;
-      sm[sw(4 * e + 2)] = v.z;
-      sm[sw(4 * e + 3)] = v.w;
+      const int at = sw(4 * e);                    // sw(4 e + j) = at ^ j
+      sm[at] = v.x;
+      sm[at ^ 1] = v.y;
+      sm[at ^ 2] = v.z;
+      sm[at ^ 3] = v.w;
     }
   } else {
     for (int e = threadIdx.x; e < len; e += kNttThreads) sm[sw(e)] = data[base + e];
@@ -257,8 +266,10 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
                      [=](int x) { return (pb5 + (x >> plane_log)) % kNP; });
   if ((len & 3) == 0) {
     uint4* dst = reinterpret_cast<uint4*>(data + base);
-    for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads)
-      dst[e] = make_uint4(sm[sw(4 * e)], sm[sw(4 * e + 1)], sm[sw(4 * e + 2)], sm[sw(4 * e + 3)]);
+    for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads) {
+      const int at = sw(4 * e);
+      dst[e] = make_uint4(sm[at], sm[at ^ 1], sm[at ^ 2], sm[at ^ 3]);
+    }
   } else {
     for (int e = threadIdx.x; e < len; e += kNttThreads) data[base + e] = sm[sw(e)];
   }
@@ -964,9 +975,16 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
 // residues of a coefficient through distributed shared memory, and a last
 // barrier keeps the CTAs resident until the others are done reading.
 
-// Threads of a cluster CTA at transform size 2^logn.
-inline int cluster_threads(int logn) {
-  return logn >= 13 ? kClusterThreadsMax : std::min(kFusedThreads, std::max(64, (1 << logn) >> 2));
+// Threads of a cluster CTA at transform size 2^logn: a quarter of the words while
+// the level's threads fit the GPU's (about 1024 per SM with these kernels'
+// registers), an eighth beyond, where whole groups of 16 words per thread cost
+// less than half-idle warps.  (Step T = 3000, S = 21: a quarter 0.292, an eighth
+// 0.306 ms; 10^4, 21: 0.550 / 0.545; 125000, 9: 2.70 / 2.64; 2^20, 9: 21.9 / 21.4.)
+inline int cluster_threads(const zr_ctx* ctx, int logn, int64_t clusters) {
+  if (logn >= 13) return kClusterThreadsMax;
+  const int64_t quarter = (int64_t)1 << (logn - 2);
+  const bool fits = clusters * kNP * quarter <= 1024ll * (ctx->sms ? ctx->sms : 152);
+  return (int)std::min<int64_t>(kFusedThreads, std::max<int64_t>(64, fits ? quarter : quarter / 2));
 }
 
 // Cluster levels go up to transforms of 2^14 (a descent CTA then holds
@@ -1794,7 +1812,7 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
     uint32_t* sp = spec[l - 1];
     const int64_t nodes = (T + (1ll << logn) - 1) >> logn;
     if (cluster_level(ctx, logn, nodes)) {
-      const cudaError_t e = launch_cluster(k_tree_cluster, nodes, cluster_threads(logn), sizeof(uint32_t) * 2 << logn,
+      const cudaError_t e = launch_cluster(k_tree_cluster, nodes, cluster_threads(ctx, logn, nodes), sizeof(uint32_t) * 2 << logn,
                                            st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M, tw, logN,
                                            l <= lspec ? (uint32_t*)nullptr : sp,
                                            (l == Lt && !root) ? (uint64_t*)nullptr : coef[l]);
@@ -2037,7 +2055,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       bool done = false;
       if (cluster_level(ctx, logn, nodes * nr)) {
         cudaEvent_t a = prof_mark(ctx, s);
-        done = launch_cluster(k_desc_cluster, nodes * nr, cluster_threads(logn), sizeof(uint32_t) * 3 << logn, s, X,
+        done = launch_cluster(k_desc_cluster, nodes * nr, cluster_threads(ctx, logn, nodes * nr), sizeof(uint32_t) * 3 << logn, s, X,
                               T, Tp, logn, C, crt_scale(logn), M, tw, logN, w.spec[l - 1], Xn, nodes) == cudaSuccess;
         if (!done) (void)cudaGetLastError();
         cudaEvent_t b2 = prof_mark(ctx, s);
@@ -2147,7 +2165,7 @@ zr_status fast_probes_enqueue(zr_ctx* ctx, int64_t G, const uint64_t* U, const u
     const int64_t nodes = (G + (1ll << logn) - 1) >> logn;
     bool done = false;
     if (cluster_level(ctx, logn, nodes * S)) {
-      done = launch_cluster(k_up_cluster, nodes * S, cluster_threads(logn), sizeof(uint32_t) * 2 << logn, st, Nc, G,
+      done = launch_cluster(k_up_cluster, nodes * S, cluster_threads(ctx, logn, nodes * S), sizeof(uint32_t) * 2 << logn, st, Nc, G,
                             Gp, logn, C, crt_scale(logn), M, tw, logN, w.spec[l - 1], Nn, nodes) == cudaSuccess;
       if (!done) (void)cudaGetLastError();
     }

@@ -60,17 +60,18 @@ __device__ __forceinline__ uint32_t mont32(uint32_t a, uint32_t b, uint32_t q, u
   const uint32_t r = hi - u;
   return (int32_t)r < 0 ? r + q : r;
 }
-__device__ __forceinline__ uint32_t sub_if(uint32_t x, uint32_t b) { return x >= b ? x - b : x; }
+__device__ __forceinline__ uint32_t sub_if(uint32_t x, uint32_t b) { return min(x, x - b); }   // x - b when x >= b
 
 // Harvey's butterflies with a Shoup twiddle: forward (CT) X, Y < 4q -> < 4q;
 // inverse (GS) X, Y < 2q -> < 2q.
+// (The sums of the forward one are written as multiply-adds: the adders issue at
+// the same rate as the multipliers and have more to do.)
 template <bool INV>
 __device__ __forceinline__ void butterfly(uint32_t& X, uint32_t& Y, uint2 w, uint32_t q) {
   if (!INV) {
     const uint32_t x = sub_if(X, 2 * q);
-    const uint32_t t = shoup32(Y, w.x, w.y, q);
-    X = x + t;
-    Y = x - t + 2 * q;
+    X = Y * w.x + x - __umulhi(Y, w.y) * q;          // x + t
+    Y = 2 * x + 2 * q - X;                           // x - t + 2 q
   } else {
     const uint32_t x = X, y = Y;
     X = sub_if(x + y, 2 * q);
@@ -84,30 +85,31 @@ __device__ __forceinline__ uint32_t residue64(uint64_t x, const NttConsts& C, in
   return shoup32(hi32(x), C.r32[i], C.r32p[i], q) + shoup32(lo32(x), 1u, C.onep[i], q);
 }
 
-// Garner: residues r_i in [0, 2q_i) (already scaled) -> the integer's residue mod p.
+// Garner: residues r_i in [0, 2q_i) (already scaled) -> the integer's residue mod
+// p.  Within a digit's steps t stays lazily below 2 q_i (y_j < q_j < 2 q_i, so
+// t + 2 q_i - y_j is in (0, 4 q_i)).
 __device__ __forceinline__ uint64_t crt_to_p(const uint32_t (&r)[kNP], const NttConsts& C, const Mod& M) {
   uint32_t y[kNP];
 #pragma unroll
   for (int i = 0; i < kNP; i++) {
     const uint32_t q = C.q[i];
-    uint32_t t = sub_if(r[i], q);
+    uint32_t t = r[i];
 #pragma unroll
-    for (int j = 0; j < i; j++) {
-      const uint32_t yj = sub_if(y[j], q);          // y_j < q_j < 2 q_i
-      t = sub_if(shoup32(t + q - yj, C.gc[i][j], C.gcp[i][j], q), q);
-    }
-    y[i] = t;
+    for (int j = 0; j < i; j++) t = shoup32(t + 2 * q - y[j], C.gc[i][j], C.gcp[i][j], q);
+    y[i] = sub_if(t, q);
   }
-  // sum_i y_i prod_{j<i} q_j, taken modulo p: y_i < 2^30, pre_i < 2^63
-  uint64_t lo = 0, hi = 0;
+  // sum_i y_i prod_{j<i} q_j, taken modulo p: y_i < 2^30, pre_i < 2^63, in 96 bits
+  uint32_t s0 = 0, s1 = 0, s2 = 0;
 #pragma unroll
-  for (int i = 0; i < kNP; i++) {
-    uint64_t ph, pl;
-    mul128(C.pre[i], (uint64_t)y[i], ph, pl);
-    lo += pl;
-    hi += ph + (lo < pl);
-  }
-  return reduce128(hi, lo, M);       // hi < 2^33 < p
+  for (int i = 0; i < kNP; i++)
+    asm("mad.lo.cc.u32 %0, %3, %5, %0;\n\t"
+        "madc.hi.cc.u32 %1, %3, %5, %1;\n\t"
+        "addc.u32 %2, %2, 0;\n\t"
+        "mad.lo.cc.u32 %1, %4, %5, %1;\n\t"
+        "madc.hi.u32 %2, %4, %5, %2;"
+        : "+r"(s0), "+r"(s1), "+r"(s2)
+        : "r"(lo32(C.pre[i])), "r"(hi32(C.pre[i])), "r"(y[i]));
+  return reduce128(s2, ((uint64_t)s1 << 32) | s0, M);       // s2 < p
 }
 
 }  // namespace zr
