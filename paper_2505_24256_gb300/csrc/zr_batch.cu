@@ -42,7 +42,7 @@ __global__ void k_b_powtab(const BDesc* __restrict__ Ds, Mod M) {
   pdl_enter();
   const BDesc& D = Ds[blockIdx.y];
   const int m = blockIdx.x, e = threadIdx.x;
-  if (D.mode == 0 && m < D.k) D.tab[m * kPowTab + e] = pow_mod(D.y[m], (uint64_t)e, M);
+  if (D.mode == 0 && D.NB > 0 && m < D.k) D.tab[m * kPowTab + e] = pow_mod(D.y[m], (uint64_t)e, M);
 }
 
 __global__ void k_b_anchor(const BDesc* __restrict__ Ds, const int64_t* __restrict__ pre, int n, Mod M) {
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kNewtonThreads) k_b_newton_table(const BDesc* 
   pdl_enter();
   extern __shared__ uint64_t tsm[];
   const BDesc& D = Ds[blockIdx.x];
-  if (D.mode != 0 || D.T == 0) return;
+  if (D.mode != 0 || D.T == 0 || D.NB == 0) return;
   newton_table_block(D.Sn, D.xs, D.invd, D.status, tsm, M);
 }
 
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kScanB) k_b_scan(const BDesc* __restrict__ Ds)
   pdl_enter();
   __shared__ int64_t sh[33];
   const BDesc& D = Ds[blockIdx.x];
-  if (D.mode != 0) return;
+  if (D.mode != 0 || D.NB == 0) return;
   const int64_t nb = (D.T + kCompB - 1) / kCompB;
   int64_t carry = 0;
   for (int64_t base = 0; base < nb; base += kScanB) {
@@ -438,6 +438,10 @@ struct Prepared {
   std::vector<int> tiles_used;        // solve instances: tile * 16 + consumer groups
   std::vector<std::vector<int4>> work;
   std::vector<char> fast;             // entries solved by the O(T log^2 T) path
+  std::vector<char> small;            // entries solved in one launch (zr_small.cu)
+  int nsmall = 0;
+  int64_t small_T = 0;                // their largest T and shared memory
+  size_t small_words = 0, o_small = 0;
   int kmax = 0, smax = 0, lmax = 0, mode = 0;
   size_t ws_bytes = 0, table_bytes = 0, fast_bytes = 0;
   int nfast = 0, fstreams = 0;        // fast entries, concurrent streams for them (0: the call's stream)
@@ -477,10 +481,23 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
   P.mode = items[0].mode;
   P.plan.resize(n);
   P.fast.assign(n, 0);
+  P.small.assign(n, 0);
   for (int i = 0; i < n; i++) {
     const BatchItem& it = items[i];
     if (it.mode != P.mode) return false;
     P.fast[i] = use_fast_solve(ctx, it.T, it.solve_S(), n) ? 1 : 0;
+    P.small[i] = !P.fast[i] && small_entry(it.T, it.solve_S(), it.S, it.k) ? 1 : 0;
+    if (P.small[i]) {
+      StepDims D = {};
+      D.T = it.T;
+      D.S = it.solve_S();
+      D.s_tile = 1;
+      P.plan[i] = D;
+      P.nsmall++;
+      P.small_T = std::max(P.small_T, it.T);
+      P.small_words = std::max(P.small_words, small_words(it.T, it.solve_S(), it.S, it.k));
+      continue;
+    }
     if (P.fast[i]) {
       // one k-block: the finish kernels read the numerators and M'(v_j) as a
       // single block's partials
@@ -501,10 +518,12 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
     P.smax = std::max(P.smax, it.S);
   }
   Carver m0(nullptr);
-  for (int i = 0; i < n; i++) carve_step(m0, items[i].T, items[i].S, items[i].k, P.plan[i], items[i].solve_S());
+  for (int i = 0; i < n; i++)
+    if (!P.small[i]) carve_step(m0, items[i].T, items[i].S, items[i].k, P.plan[i], items[i].solve_S());
   P.ws_bytes = m0.off;
   std::vector<int64_t> c_hash(n), c_roots(n), c_leaf(n), c_carry(n), c_nblk(n);
   for (int i = 0; i < n; i++) {
+    if (P.small[i]) continue;
     const int64_t T = items[i].T;
     c_hash[i] = T > 0 ? (int64_t)hash_slots(T) : 0;
     c_roots[i] = T;
@@ -517,16 +536,19 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
   push_prefix(P.pre, c_leaf, P.o_leaf);
   push_prefix(P.pre, c_carry, P.o_carry);
   push_prefix(P.pre, c_nblk, P.o_nblk);
+  P.o_small = P.pre.size();
+  for (int i = 0; i < n; i++)
+    if (P.small[i]) P.pre.push_back(i);
   for (int l = kTreeL1; l < P.lmax; l++) {
     std::vector<int64_t> c(n);
     for (int i = 0; i < n; i++)
-      c[i] = (!P.fast[i] && tree_levels(items[i].T) > l) ? (items[i].T + tree_tile(l) - 1) / tree_tile(l) : 0;
+      c[i] = (!P.fast[i] && !P.small[i] && tree_levels(items[i].T) > l) ? (items[i].T + tree_tile(l) - 1) / tree_tile(l) : 0;
     size_t o;
     push_prefix(P.pre, c, o);
     P.o_lvl.push_back(o);
   }
   for (int i = 0; i < n; i++) {
-    if (items[i].T == 0 || P.fast[i]) continue;
+    if (items[i].T == 0 || P.fast[i] || P.small[i]) continue;
     // one work list per (tile, consumer groups): the solve kernel instance
     const int tile = P.plan[i].s_tile, groups = (items[i].solve_S() + tile - 1) / tile;
     const int key = tile * 16 + groups;
@@ -547,7 +569,7 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
     });
   P.table_bytes = sizeof(BDesc) * n + sizeof(int64_t) * P.pre.size();
   for (auto& wl : P.work) P.table_bytes += sizeof(int4) * wl.size() + 16;
-  P.fstreams = (P.nfast >= 2 || (P.nfast >= 1 && P.nfast < n)) ? std::min(P.nfast, kFastStreams) : 0;
+  P.fstreams = (P.nfast >= 2 || (P.nfast >= 1 && P.nfast + P.nsmall < n)) ? std::min(P.nfast, kFastStreams) : 0;
   P.fast_bytes = P.nfast ? P.fast_slot * (size_t)std::max(P.fstreams, 1) : 0;
   return true;
 }
@@ -589,7 +611,8 @@ static zr_status stage_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_
   Carver cv(ws);
   for (int i = 0; i < n; i++) {
     const BatchItem& it = items[i];
-    StepWs w = carve_step(cv, it.T, it.S, it.k, plan[i], it.solve_S());
+    StepWs w = {};
+    if (!P.small[i]) w = carve_step(cv, it.T, it.S, it.k, plan[i], it.solve_S());
     const bool given0 = it.solve_S() != it.S;
     BDesc& d = D[i];
     memset(&d, 0, sizeof(d));
@@ -707,10 +730,18 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
   const int64_t ncarry = pre[o_carry + n];
   // entries with T = 0 report an empty skeleton
   for (int64_t* c : SB.zero_counts) cudaMemsetAsync(c, 0, 8, st);
+  if (P.nsmall && !nroots) {
+    // small entries only: one launch
+    cudaEvent_t a = mark();
+    const cudaError_t e = launch_small(dD, dpre + P.o_small, P.nsmall, P.small_T, P.small_words, M, st);
+    cudaEvent_t b = mark();
+    prof_add(ctx, PH_SOLVE, a, b);
+    return cuda_err(ctx, e != cudaSuccess ? e : cudaGetLastError(), "small steps");
+  }
   // Newton's matrix W depends only on the samples: build it on the side
   // stream while the tree, carries and solve run (joined before the finish)
   bool side = false;
-  if (mode == 0 && nroots) {
+  if ((mode == 0 || P.nsmall) && nroots) {
     if (!ctx->side) cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
     if (!ctx->ev_fork) cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
     if (!ctx->ev_join) cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
@@ -718,10 +749,20 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       configure_newton_kernels();
       cudaEventRecord(ctx->ev_fork, st);
       cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
-      launch_k(k_b_newton_table, n, kNewtonThreads, 8 * (size_t)newton_table_words(smax), ctx->side, dD, M);
-      note_launch();
+      if (mode == 0) {
+        launch_k(k_b_newton_table, n, kNewtonThreads, 8 * (size_t)newton_table_words(smax), ctx->side, dD, M);
+        note_launch();
+      }
+      // small entries beside the others (their samples' matrices are their own)
+      if (P.nsmall) {
+        const cudaError_t e = launch_small(dD, dpre + P.o_small, P.nsmall, P.small_T, P.small_words, M, ctx->side);
+        if (e != cudaSuccess) return cuda_err(ctx, e, "small steps");
+      }
       cudaEventRecord(ctx->ev_join, ctx->side);
       side = true;
+    } else if (P.nsmall) {
+      const cudaError_t e = launch_small(dD, dpre + P.o_small, P.nsmall, P.small_T, P.small_words, M, st);
+      if (e != cudaSuccess) return cuda_err(ctx, e, "small steps");
     }
   }
   cudaEvent_t e0 = mark();
@@ -774,7 +815,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
     const int64_t want = 4ll * (ctx->sms ? ctx->sms : 152);
     int split = (int)((want + nt - 1) / nt);
     for (int i = 0; i < n; i++)
-      if (!P.fast[i] && tree_levels(P.plan[i].T) > l) split = std::min(split, (int)tree_split_max(P.plan[i].T));
+      if (!P.fast[i] && !P.small[i] && tree_levels(P.plan[i].T) > l) split = std::min(split, (int)tree_split_max(P.plan[i].T));
     // and keep at least 128 inner terms per split: below that the combine
     // launch costs more than the shorter serial work saves
     split = std::min(split, (int)std::max<int64_t>(1, (1ll << l) / 128));
@@ -828,6 +869,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       }
     } else {
       { launch_k(k_b_finish_solve, cdiv(nroots, 256), 256, 0, st, dD, dpre + o_roots, n, M); note_launch(); }
+      if (side) cudaStreamWaitEvent(st, ctx->ev_join, 0);   // the small entries (forked above)
     }
   }
   cudaEvent_t e5 = mark();

@@ -161,6 +161,13 @@ struct BatchItem {
   const uint64_t* c0 = nullptr;
   int solve_S() const { return c0 && mode == 0 && S >= 2 ? S - 1 : S; }
 };
+// Small entries (zr_small.cu), solved in one launch: whether an entry of T
+// unknowns, S systems, Sn samples and k variables is one, the shared memory
+// words it needs, and the launch of the n entries idx[0..n) of Ds.
+bool small_entry(int64_t T, int S, int Sn, int k);
+size_t small_words(int64_t T, int S, int Sn, int k);
+cudaError_t launch_small(const BDesc* Ds, const int64_t* idx, int n, int64_t Tmax, size_t words, const Mod& M,
+                         cudaStream_t st);
 // Workspace bytes a batch needs (its regions plus the device tables).
 size_t batch_ws_need(const zr_ctx* ctx, const BatchItem* items, int n);
 // Enqueues a batch; its workspace starts `base` bytes into the context

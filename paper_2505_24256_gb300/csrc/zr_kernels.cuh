@@ -81,7 +81,7 @@ struct StepDims {
 struct BDesc {
   int64_t T, BK, ldb, ldc, out_cap;
   uint64_t hmask;
-  int32_t S, k, nv, offset, mode, NB, s_tile, nst, levels;
+  int32_t S, k, nv, offset, mode, NB, s_tile, nst, levels;   // NB = 0: a small entry (zr_small.cu)
   int32_t Sn;   // samples interpolated: S (systems solved), or S + 1 with c0
   const uint8_t* exps;
   const uint64_t *y, *xs, *b;
