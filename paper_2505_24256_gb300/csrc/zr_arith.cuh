@@ -168,8 +168,46 @@ __device__ __forceinline__ uint64_t pow_mod(uint64_t a, uint64_t e, const Mod& M
   }
   return r;
 }
-// Inverse by Fermat's little theorem (p prime); 0 maps to 0.
-__device__ __forceinline__ uint64_t inv_mod(uint64_t a, const Mod& M) { return pow_mod(a, M.p - 2, M); }
+// Inverse of a < p modulo the odd prime p; 0 maps to 0.  Kaliski's almost
+// Montgomery inverse ("The Montgomery inverse and its applications", IEEE
+// Trans. Computers 44(8), 1995) with whole runs of shifts at a time, then the
+// shifts undone by Montgomery reductions.  Invariants: p = u s + v r, a r = -u
+// 2^k and a s = v 2^k (mod p), u and v odd; u = v = 1 at the end, so a^-1 = s
+// 2^-k, and r, s stay below p.  About 44 subtractions of 50 cycles and two
+// reductions; a power to p - 2 is 63 squarings of 170 to 320 cycles in sequence
+// (a third of a small step's time: 20000 cycles, against 5000).
+__device__ __forceinline__ uint64_t inv_mod(uint64_t a, const Mod& M) {
+  if (a == 0) return 0;
+  int k = __ffsll((long long)a) - 1;
+  uint64_t u = M.p, v = a >> k, r = 0, s = 1;
+  while (u != v) {
+    const bool ug = u > v;
+    const uint64_t diff = ug ? u - v : v - u, sum = r + s;
+    const int t = __ffsll((long long)diff) - 1;
+    const uint64_t kept = (ug ? s : r) << t;
+    u = ug ? diff >> t : u;
+    v = ug ? v : diff >> t;
+    r = ug ? sum : kept;
+    s = ug ? kept : sum;
+    k += t;
+  }
+  uint64_t pinv = M.p;                           // p^-1 mod 2^64: p is its own inverse mod 8
+#pragma unroll
+  for (int i = 0; i < 5; i++) pinv *= 2 - M.p * pinv;
+  // s 2^-t for t < 64: (s + (-s p^-1 mod 2^t) p) / 2^t
+  auto halve = [&](uint64_t x, int t) -> uint64_t {
+    if (t == 0) return x;
+    const uint64_t q = (0 - x * pinv) & ((1ull << t) - 1);
+    uint64_t hi, lo;
+    mul128(q, M.p, hi, lo);
+    lo += x;
+    hi += lo < x;
+    return (hi << (64 - t)) | (lo >> t);
+  };
+  const int t1 = k < 63 ? k : 63;
+  const uint64_t x = halve(s, t1);
+  return canon(halve(x, k - t1), M);
+}
 
 // ---------------------------------------------------------------------------
 // Deferred multiply-accumulate: acc += x b for 64-bit x, b, reduced once.
