@@ -112,8 +112,8 @@ zr_status zr_check_bounded_wait(zr_ctx* ctx, uint32_t tries, void* stream);
  *   6 dot         out[i] = sum_{t < len} a[i len + t] b[i len + t] mod p
  *                 (1 <= len < 2^31; one 160-bit accumulator per i)
  *   7 add, 8 sub  out = a +- b mod p                             (a, b < p)
- *   9 batch_inv   out = a^-1 mod p (0 for a = 0) by Montgomery's batch trick
- *                 over consecutive groups of 32
+ *   9 batch_inv   out = a^-1 mod p (0 for a = 0), the steps' inversion of the
+ *                 denominators of 32 consecutive roots by a warp
  * a, b, out: device arrays (b unused by 2, 5, 9); for dot, a and b hold
  * n len values.  hits: NULL, or a device uint32[4] to which the call adds how
  * often the two correction steps of the Moller-Granlund division ran

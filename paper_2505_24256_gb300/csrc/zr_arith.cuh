@@ -234,6 +234,21 @@ __device__ __forceinline__ void mac8(Acc8& a, uint32_t x0, uint32_t x1, uint32_t
       : "+r"(a.r0), "+r"(a.r1), "+r"(a.r2), "+r"(a.r3), "+r"(a.r4), "+r"(a.t0), "+r"(a.t1), "+r"(a.t2)
       : "r"(x0), "r"(x1), "r"(b0), "r"(b1));
 }
+// a += b
+__device__ __forceinline__ void acc8_add(Acc8& a, const Acc8& b) {
+  asm("add.cc.u32 %0, %0, %5;\n\t"
+      "addc.cc.u32 %1, %1, %6;\n\t"
+      "addc.cc.u32 %2, %2, %7;\n\t"
+      "addc.cc.u32 %3, %3, %8;\n\t"
+      "addc.u32 %4, %4, %9;"
+      : "+r"(a.r0), "+r"(a.r1), "+r"(a.r2), "+r"(a.r3), "+r"(a.r4)
+      : "r"(b.r0), "r"(b.r1), "r"(b.r2), "r"(b.r3), "r"(b.r4));
+  asm("add.cc.u32 %0, %0, %3;\n\t"
+      "addc.cc.u32 %1, %1, %4;\n\t"
+      "addc.u32 %2, %2, %5;"
+      : "+r"(a.t0), "+r"(a.t1), "+r"(a.t2)
+      : "r"(b.t0), "r"(b.t1), "r"(b.t2));
+}
 // residue of r + t 2^32
 __device__ __forceinline__ uint64_t acc8_value(const Acc8& a, const Mod& M) {
   const uint64_t L = ((uint64_t)a.r1 << 32) | a.r0;

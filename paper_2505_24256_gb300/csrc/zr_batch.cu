@@ -12,7 +12,7 @@
 //   anchor values v_j and the distinctness check (hash table)      a2
 //   master polynomial by a product tree                             a3
 //   k-block carries, then the synthetic-division / dot kernel       a4, a5
-//   denominators, Montgomery batch inversion, Newton, counts        a4, a6
+//   denominators, their inverses, Newton, counts                    a4, a6
 //   compaction of the new skeleton                                  a6
 #include <cuda_runtime.h>
 
@@ -234,16 +234,15 @@ __device__ __forceinline__ uint64_t root_den(const BDesc& D, int64_t j, uint64_t
 
 // W of every step entry (one block each): the values -> monomial map of Newton
 // interpolation on the entry's S samples.
-__global__ void __launch_bounds__(kNewtonThreads) k_b_newton_table(const BDesc* __restrict__ Ds, Mod M) {
+__global__ void __launch_bounds__(32) k_b_newton_table(const BDesc* __restrict__ Ds, Mod M) {
   pdl_enter();
-  extern __shared__ uint64_t tsm[];
   const BDesc& D = Ds[blockIdx.x];
   if (D.mode != 0 || D.T == 0 || D.NB == 0) return;
-  newton_table_block(D.Sn, D.xs, D.invd, D.status, tsm, M);
+  newton_matrix(D.Sn, D.xs, D.invd, D.status, M);
 }
 
 // a4 + a6 per term: the denominator q_j(v_j) from its k-block partials, its
-// inverse (one inversion per warp), the S dot products from their k-block
+// inverse, the S dot products from their k-block
 // partials, then the monomial coefficients through W.  Blocks of kFinB terms
 // never straddle entries (pre counts blocks), so W sits in shared memory.
 // kFinSplit warps share a block: the first inverts, all sum the partials of
@@ -702,8 +701,6 @@ static zr_status stage_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_
 static void configure_newton_kernels() {
   static DeviceOnce attr;
   attr.run([] {
-    cudaFuncSetAttribute(k_b_newton_table, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(8 * newton_table_words(kNewtonMax)));
     cudaFuncSetAttribute(k_b_finish_newton, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)newton_smem(kNewtonMax, kFinB));
   });
@@ -750,7 +747,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       cudaEventRecord(ctx->ev_fork, st);
       cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
       if (mode == 0) {
-        launch_k(k_b_newton_table, n, kNewtonThreads, 8 * (size_t)newton_table_words(smax), ctx->side, dD, M);
+        launch_k(k_b_newton_table, n, 32, 0, ctx->side, dD, M);
         note_launch();
       }
       // small entries beside the others (their samples' matrices are their own)
@@ -858,7 +855,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       configure_newton_kernels();
       if (side) cudaStreamWaitEvent(st, ctx->ev_join, 0);   // W of every entry (forked above)
       else {
-        launch_k(k_b_newton_table, n, kNewtonThreads, 8 * (size_t)newton_table_words(smax), st, dD, M);
+        launch_k(k_b_newton_table, n, 32, 0, st, dD, M);
         note_launch();
       }
       const int64_t nblk = pre[o_nblk + n];

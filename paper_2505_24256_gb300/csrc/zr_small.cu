@@ -8,10 +8,11 @@
 //   every CTA    the anchor values of all T terms and the master polynomial by
 //                the product tree (short enough to repeat, so that nothing is
 //                exchanged);
-//   warps 0-7    lane = root, warp = k-block: the block's Horner value, the
+//   warps 0-15   lane = root, warp = k-block: the block's Horner value, the
 //                carry from the blocks above, the quotients q_k with their Horner
-//                value, then the block's part of every dot product;
-//   warp 8       lane = sample: the values -> monomials matrix of Newton's
+//                value; then a warp per right-hand side and part of k: the dot
+//                products;
+//   warp 16      lane = sample: the values -> monomials matrix of Newton's
 //                interpolation, beside all that;
 //   then         the sums over the blocks, one inverse, Newton, and the compaction
 //                (the CTAs' counts through distributed shared memory).
@@ -32,16 +33,17 @@ namespace zr {
 namespace {
 
 constexpr int kSmRoots = 32;                     // roots of a CTA: a lane each
-constexpr int kSmWarps = 8;                      // k-blocks
+constexpr int kSmWarps = 16;                     // k-blocks
 constexpr int kSmThreads = 32 * (kSmWarps + 1);
 
 struct SmallSmem {
   // word offsets of the dynamic shared memory
   int v, tree, tab, b, q, part, num, W, total;
 };
+// parts of k a dot product is split into: two or three items a warp
+__host__ __device__ inline int small_parts(int S) { return S >= 2 * kSmWarps ? 1 : (2 * kSmWarps + S - 1) / S; }
 __host__ __device__ inline SmallSmem small_smem(int T, int S, int Sn, int k) {
   SmallSmem o;
-  const int BK = (T + kSmWarps - 1) / kSmWarps;
   int at = 0;
   o.v = at;
   at += T;
@@ -52,9 +54,9 @@ __host__ __device__ inline SmallSmem small_smem(int T, int S, int Sn, int k) {
   o.b = at;
   at += S * T;
   o.q = at;                                      // the quotients, later the coefficients
-  at += (kSmWarps * BK > Sn ? kSmWarps * BK : Sn) * kSmRoots;
+  at += (T > Sn ? T : Sn) * kSmRoots;
   o.part = at;
-  at += kSmWarps * S * kSmRoots;
+  at += small_parts(S) * S * kSmRoots;
   o.num = at;
   at += Sn * kSmRoots;
   o.W = at;
@@ -63,13 +65,40 @@ __host__ __device__ inline SmallSmem small_smem(int T, int S, int Sn, int k) {
   return o;
 }
 
-__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+constexpr int kSmMain = 32 * kSmWarps;
+__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSmMain) : "memory"); }
+
+// Coefficient n of (A + z^a)(B + z^b), below z^(a+b), A at in[0..a), B at
+// in[a..a+b): half h of the products by each of two neighbouring lanes, in two
+// sums (a chain of multiply-adds takes 50 cycles a product).
+__device__ __forceinline__ uint64_t conv_half(const uint64_t* in, int a, int b, int n, int h, const Mod& M) {
+  const int lo = max(0, n - b + 1), hi = min(a - 1, n) + 1, mid = lo + (max(hi - lo, 0) >> 1);
+  const int i0 = h ? mid : lo, i1 = h ? hi : mid;
+  Acc8 s0 = {0, 0, 0, 0, 0, 0, 0, 0}, s1 = {0, 0, 0, 0, 0, 0, 0, 0};
+  const uint64_t* B = in + a + n;
+  int i = i0;
+#pragma unroll 2
+  for (; i + 1 < i1; i += 2) {
+    const uint64_t x = in[i], y = B[-i], z = in[i + 1], w = B[-i - 1];
+    mac8(s0, lo32(x), hi32(x), lo32(y), hi32(y));
+    mac8(s1, lo32(z), hi32(z), lo32(w), hi32(w));
+  }
+  if (i < i1) {
+    const uint64_t x = in[i], y = B[-i];
+    mac8(s0, lo32(x), hi32(x), lo32(y), hi32(y));
+  }
+  acc8_add(s0, s1);
+  uint64_t r = acc8_value(s0, M);
+  if (h == 0 && n >= a) r = add_mod(r, in[n], M);            // z^a times B_{n-a}
+  if (h == 1 && n >= b) r = add_mod(r, in[n - b], M);        // z^b times A_{n-b}
+  return r;
+}
 
 __global__ void __launch_bounds__(kSmThreads, 1)
     k_small(const BDesc* __restrict__ Ds, const int64_t* __restrict__ idx, int cl, Mod M) {
   pdl_enter();
   extern __shared__ uint64_t ssm[];
-  __shared__ uint64_t rs[kSmWarps][kSmRoots], us[kSmWarps][kSmRoots], invs[kSmRoots];
+  __shared__ uint64_t sq[kMaxVars][8], rs[kSmWarps][kSmRoots], us[kSmWarps][kSmRoots], invs[kSmRoots];
   __shared__ uint32_t nz[32], masks[kSmRoots];
   __shared__ int offs[kSmRoots], tot[8];
   asm volatile("barrier.cluster.arrive;" ::: "memory");   // waited for before another CTA's memory is written
@@ -84,40 +113,31 @@ __global__ void __launch_bounds__(kSmThreads, 1)
   const bool live = j < T, any = j0 < T;         // CTAs past the entry's roots only count
   const unsigned FULL = 0xffffffffu;
   const int BK = (T + kSmWarps - 1) / kSmWarps, wl = (T - 1) / BK;   // the last block that holds anything
+  const int kp = small_parts(S);
 
   if (warp == kSmWarps) {
-    if (D.mode == 0 && any) {
-      // W[e][s] = coefficient e of prod_{t != s} (z - x_t) / (x_s - x_t):
-      // P = prod (z - x_t), lane e its coefficient; then lane s divides by z - x_s
-      const uint64_t x = lane < Sn ? D.xs[lane] : 0, xq = shoup_pre(x, M);
-      uint64_t c = lane == 0 ? 1 : 0;
-      for (int t = 0; t < Sn; t++) {
-        uint64_t up = __shfl_up_sync(FULL, c, 1);
-        if (lane == 0) up = 0;
-        c = sub_mod(up, mul_mod(__shfl_sync(FULL, x, t), c, M), M);
-      }
-      uint64_t q = 1, u = 0;
-      for (int e = Sn - 1; e >= 0; e--) {
-        u = add_mod(canon(shoup_lazy(u, x, xq, M), M), q, M);
-        if (lane < Sn) W[e * Sn + lane] = q;
-        q = add_mod(canon(shoup_lazy(q, x, xq, M), M), __shfl_sync(FULL, c, e), M);
-      }
-      if (lane < Sn && u == 0 && rank == 0) atomicOr(D.status, ST_DUP_SAMPLE);
-      const uint64_t inv = warp_batch_inverse(lane < Sn ? u : 1, M);
-      if (lane < Sn)
-        for (int e = 0; e < Sn; e++) W[e * Sn + lane] = mul_mod(W[e * Sn + lane], inv, M);
-    }
+    if (D.mode == 0 && any) newton_matrix_warp<1>(Sn, D.xs, W, rank == 0 ? D.status : nullptr, M);
   } else if (any) {
     // the right-hand sides, on their way while the nodes are made
-    for (int i = tid; i < S * T; i += 256) {
-      const int s = i / T;
-      cp_async8(bs + i, D.b + (int64_t)s * D.ldb + (i - s * T));
-    }
+    for (int s = 0; s < S; s++)
+      if (tid < T) cp_async8(bs + s * T + tid, D.b + (int64_t)s * D.ldb + tid);
     cp_async_commit();
-    // anchor values
-    for (int i = tid; i < 32 * k; i += 256) {
-      const int m = i >> 5, e = i & 31;
-      tab[i] = pow_mod(D.y[m], e < 16 ? e : (uint64_t)(e - 16) * 16, M);
+    // anchor powers: x^(2^b), then x^e and x^(16 e), e < 16, from them
+    if (tid < k) {
+      uint64_t x = D.y[tid];
+      for (int b = 0; b < 8; b++) {
+        sq[tid][b] = x;
+        x = mul_mod(x, x, M);
+      }
+    }
+    main_sync();
+    for (int i = tid; i < 32 * k; i += kSmMain) {
+      const uint64_t* b = sq[i >> 5] + ((i >> 2) & 4);
+      uint64_t x = i & 1 ? b[0] : 1;
+#pragma unroll
+      for (int q = 1; q < 4; q++)
+        if ((i >> q) & 1) x = mul_mod(x, b[q], M);
+      tab[i] = x;
     }
     main_sync();
     if (tid < T) {
@@ -139,22 +159,37 @@ __global__ void __launch_bounds__(kSmThreads, 1)
       }
       if (D.offset == 1 && x == 0) atomicOr(D.status, ST_ZERO_NODE);
       vs[tid] = x;
-      tree[tid] = x ? M.p - x : 0;               // z - v_j
     }
     main_sync();
-    // M's coefficients below its leading 1
-    uint64_t *in = tree, *out = tree + T;
-    for (int size = 1; size < T; size *= 2) {
-      if (tid < T) {
-        const int po = tid & ~(2 * size - 1);
-        out[tid] = T - po <= size ? in[tid] : conv_coef(in, po, size, min(size, T - po - size), tid - po, M);
+    // M's coefficients below its leading 1: blocks of 32 roots, a factor at a
+    // time with the coefficients in a warp's lanes (half the time of the tree's
+    // first five levels), then pairs, two lanes a coefficient
+    if (32 * warp < T) {
+      const uint64_t x = tid < T ? vs[tid] : 0, xq = shoup_pre(x, M);
+      uint64_t c = lane == 0 ? 1 : 0;
+      for (int t = 0; t < min(32, T - 32 * warp); t++) {
+        uint64_t up = __shfl_up_sync(FULL, c, 1);
+        if (lane == 0) up = 0;
+        const uint64_t xt = __shfl_sync(FULL, x, t), xqt = __shfl_sync(FULL, xq, t);
+        c = sub_mod(up, canon(shoup_lazy(c, xt, xqt, M), M), M);
       }
+      if (tid < T) tree[tid] = c;
+    }
+    main_sync();
+    int in = o.tree, out = o.tree + T;
+    for (int size = 32; size < T; size *= 2) {
+      const int n = tid >> 1, h = tid & 1, po = n & ~(2 * size - 1);
+      uint64_t x = 0;
+      const bool pair = n < T && T - po > size;
+      if (pair) x = conv_half(ssm + in + po, size, min(size, T - po - size), n - po, h, M);
+      x = add_mod(x, __shfl_xor_sync(FULL, x, 1), M);
+      if (n < T && h == 0) ssm[out + n] = pair ? x : ssm[in + n];
       main_sync();
-      uint64_t* t = in;
+      const int t = in;
       in = out;
       out = t;
     }
-    const uint64_t* m = in;
+    const uint64_t* m = ssm + in;
     // k-blocks [klo, khi): the block's Horner value (the last one's includes m_T
     // = 1), the carry from the blocks above, the quotients
     const uint64_t v = live ? vs[j] : 0, vq = shoup_pre(v, M);
@@ -166,7 +201,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     main_sync();
     uint64_t q = warp == wl ? 1 : 0, u = 0;
     for (int w = wl; w > warp; w--) q = add_mod(canon(shoup_lazy(q, vBK, vBKq, M), M), rs[w][lane], M);
-    uint64_t* qw = qs + warp * BK * kSmRoots + lane;
+    uint64_t* qw = qs + klo * kSmRoots + lane;
     for (int i = khi - 1; i >= klo; i--) {
       const uint64_t qc = canon(q, M);
       qw[(i - klo) * kSmRoots] = qc;
@@ -176,27 +211,25 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     us[warp][lane] = canon(u, M);
     cp_async_wait<0>();
     main_sync();
-    // the block's part of the dot products, four right-hand sides at a time
-    for (int s0 = 0; s0 < S; s0 += 4) {
-      Acc8 acc[4];
-      const uint64_t* row[4];
-#pragma unroll
-      for (int c = 0; c < 4; c++) {
-        acc[c] = Acc8{0, 0, 0, 0, 0, 0, 0, 0};
-        row[c] = bs + min(s0 + c, S - 1) * T;
+    // dot products: a warp takes right-hand side s and the p-th of kp parts of k
+    for (int it = warp; it < S * kp; it += kSmWarps) {
+      const int p = it / S, s = it - p * S;
+      const int k0 = T * p / kp, k1 = T * (p + 1) / kp;
+      Acc8 a0 = {0, 0, 0, 0, 0, 0, 0, 0}, a1 = {0, 0, 0, 0, 0, 0, 0, 0};
+      const uint64_t *x = qs + lane, *w = bs + s * T;
+      int i = k0;
+#pragma unroll 2
+      for (; i + 1 < k1; i += 2) {
+        const uint64_t x0 = x[i * kSmRoots], x1 = x[(i + 1) * kSmRoots], w0 = w[i], w1 = w[i + 1];
+        mac8(a0, lo32(x0), hi32(x0), lo32(w0), hi32(w0));
+        mac8(a1, lo32(x1), hi32(x1), lo32(w1), hi32(w1));
       }
-#pragma unroll 4
-      for (int i = klo; i < khi; i++) {
-        const uint64_t x = qw[(i - klo) * kSmRoots];
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-          const uint64_t w = row[c][i];
-          mac8(acc[c], lo32(x), hi32(x), lo32(w), hi32(w));
-        }
+      if (i < k1) {
+        const uint64_t x0 = x[i * kSmRoots], w0 = w[i];
+        mac8(a0, lo32(x0), hi32(x0), lo32(w0), hi32(w0));
       }
-#pragma unroll
-      for (int c = 0; c < 4; c++)
-        if (s0 + c < S) part[(warp * S + s0 + c) * kSmRoots + lane] = acc8_value(acc[c], M);
+      acc8_add(a0, a1);
+      part[it * kSmRoots + lane] = acc8_value(a0, M);
     }
     main_sync();
     if (warp == 0) {
@@ -208,7 +241,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     } else {
       for (int s = warp - 1; s < S; s += kSmWarps - 1) {
         uint64_t x = 0;
-        for (int w = 0; w <= wl; w++) x = add_mod(x, part[(w * S + s) * kSmRoots + lane], M);
+        for (int p = 0; p < kp; p++) x = add_mod(x, part[(p * S + s) * kSmRoots + lane], M);
         num[(s + s1) * kSmRoots + lane] = x;
       }
     }
@@ -295,7 +328,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
   }
 }
 
-constexpr size_t kSmMaxSmem = 216 * 1024;
+constexpr size_t kSmMaxSmem = 208 * 1024;   // beside 13 KB of static arrays
 
 // whether this device runs clusters of eight with the largest shared memory
 bool small_supported() {

@@ -75,23 +75,16 @@ void launch_node_check(int64_t T, const uint64_t* v, uint64_t* htab, uint64_t hm
 
 // ---------------------------------------------------------------------------
 // a6: Newton in the new variable, Eq. (newton).
-//   invd[l S + s] = 1 / (x_s - x_{s-l}),  1 <= l <= s < S   (shared by all terms)
+//   W: values -> monomial coefficients (shared by all terms)
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(kNewtonThreads) k_newton_table(int S, const uint64_t* __restrict__ xs, Mod M,
-                                                                  uint64_t* __restrict__ W, uint32_t* status) {
-  extern __shared__ uint64_t tsm[];
-  newton_table_block(S, xs, W, status, tsm, M);
+__global__ void __launch_bounds__(32) k_newton_table(int S, const uint64_t* __restrict__ xs, Mod M,
+                                                     uint64_t* __restrict__ W, uint32_t* status) {
+  newton_matrix(S, xs, W, status, M);
 }
 
 void launch_newton_table(int S, const uint64_t* xs, const Mod& M, uint64_t* W, uint32_t* status, cudaStream_t st) {
-  static DeviceOnce attr;
-  attr.run([] {
-    cudaFuncSetAttribute(k_newton_table, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(8 * newton_table_words(kNewtonMax)));
-  });
-  const size_t smem = 8 * (size_t)newton_table_words(S);
-  { k_newton_table<<<1, kNewtonThreads, smem, st>>>(S, xs, M, W, status); note_launch(); }
+  { k_newton_table<<<1, 32, 0, st>>>(S, xs, M, W, status); note_launch(); }
 }
 
 // One block of 128 terms: the block's values and W in shared memory, then

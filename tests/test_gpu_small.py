@@ -112,3 +112,13 @@ def test_small_failures(ctx, orc, T):
     d, keep, ref = step(ctx, 5 * T, T, 3, 2, 20, 0)
     ctx.zippel_step_batched([d])
     check(orc, d, ref)
+
+
+def test_small_step_is_one_launch(ctx, orc):
+    from paper_2505_24256_gb300 import zr
+
+    d, keep, ref = step(ctx, 9, 256, 21, 5, 20, 0)
+    before = zr.launch_count()
+    ctx.zippel_step_batched([d])
+    assert zr.launch_count() - before == 1
+    check(orc, d, ref)
