@@ -369,11 +369,10 @@ extern "C" zr_status zr_create(uint64_t prime, zr_ctx** out) {
   ctx->ntt = make_ntt_consts(prime);
   cudaError_t e = cudaGetDevice(&ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device);
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, 2 * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, 2 * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, 2 * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_count, 4 * sizeof(int64_t));
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_count, 4 * sizeof(int64_t));
+  const size_t words = 2 * sizeof(uint32_t) + 4 * sizeof(int64_t);   // two status words, four counts
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, words);
+  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, words);
+  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, words);
   if (e == cudaSuccess) {
     // reconstructions allocate their per-request buffers from the device's
     // pool in stream order; keep freed blocks in the pool for the next ones
@@ -389,6 +388,8 @@ extern "C" zr_status zr_create(uint64_t prime, zr_ctx** out) {
     return e == cudaErrorMemoryAllocation ? ZR_ERR_OOM : ZR_ERR_CUDA;
   }
   ctx->d_status_call = ctx->d_status + 1;
+  ctx->d_count = reinterpret_cast<int64_t*>(ctx->d_status + 2);
+  ctx->h_count = reinterpret_cast<int64_t*>(ctx->h_status + 2);
   *out = ctx;
   return ZR_OK;
 }
@@ -400,8 +401,6 @@ extern "C" void zr_destroy(zr_ctx* ctx) {
   if (ctx->ws) cudaFree(ctx->ws);
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
-  if (ctx->d_count) cudaFree(ctx->d_count);
-  if (ctx->h_count) cudaFreeHost(ctx->h_count);
   if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
   if (ctx->stage_event) cudaEventDestroy(ctx->stage_event);
   if (ctx->side) cudaStreamDestroy(ctx->side);
@@ -514,11 +513,14 @@ extern "C" zr_status zr_solve_method(zr_ctx* ctx, int32_t method, int64_t crosso
 extern "C" uint64_t zr_prime(const zr_ctx* ctx) { return ctx ? ctx->M.p : 0; }
 extern "C" size_t zr_workspace_bytes(const zr_ctx* ctx) { return ctx ? ctx->ws_cap : 0; }
 
+cudaError_t zr::read_call_status(zr_ctx* ctx, int counts, cudaStream_t st) {
+  return cudaMemcpyAsync(ctx->h_status + 1, ctx->d_status_call, sizeof(uint32_t) + counts * sizeof(int64_t),
+                         cudaMemcpyDeviceToHost, st);
+}
+
 // Reads and clears the per-call status word after the stream drains.
 static zr_status finish_sync_call(zr_ctx* ctx, cudaStream_t st, int64_t* count_out) {
-  cudaError_t e = cudaMemcpyAsync(ctx->h_status + 1, ctx->d_status_call, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && count_out)
-    e = cudaMemcpyAsync(ctx->h_count, ctx->d_count, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+  cudaError_t e = read_call_status(ctx, count_out ? 1 : 0, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_err(ctx, e, "synchronise");
   e = cudaGetLastError();

