@@ -360,70 +360,165 @@ __global__ void k_tree_crt(const uint32_t* __restrict__ Z, int64_t T, int64_t Tp
   coef[r] = x;
 }
 
-// Descent load: XH[r][i][P n + k] = X_P[d_P - 1 - k] (k < d_P), else 0; one
-// thread per (r, P n + k) writes all five primes' residues.
-__global__ void k_desc_load(const uint64_t* __restrict__ X, int R, int64_t T, int64_t Tp, int logn, NttConsts C,
-                            uint32_t* __restrict__ XH) {
-  pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over R * T'
-  if (idx >= (int64_t)R * Tp) return;
-  const int rr = (int)(idx / Tp);
-  const int64_t e = idx - (int64_t)rr * Tp;
-  const int64_t n = 1ll << logn;
-  const int64_t P = e >> logn, k = e & (n - 1);
-  int64_t d = T - P * n;
-  d = d < 0 ? 0 : (d > n ? n : d);
-  const uint64_t x = k < d ? X[(int64_t)rr * Tp + P * n + d - 1 - k] : 0;
-  uint32_t* out = XH + (int64_t)rr * kNP * Tp + e;
-#pragma unroll
-  for (int i = 0; i < kNP; i++) out[(int64_t)i * Tp] = k < d ? residue64(x, C, i) : 0u;
+// ---- descent levels of large transforms --------------------------------------------
+//
+// A level of transforms n = 2^logn >= 2^13 (L1 = logn - 13) takes three kernels:
+// the first L1 forward stages on columns, straight from the expansions; per
+// tile of 2^13 words the other forward stages, both products and the inverse
+// stages that stay inside it; the last L1 inverse stages on columns, with the
+// Chinese remaindering.  (Loads, products and remaindering as passes of their
+// own moved 17 + 4 words of 20 bytes per coefficient, now 6 + 1.)  A node whose
+// right child holds no roots (R = 1) is copied: X_L[m] = X_P[m].
+
+constexpr int kTileThreads = 512;              // k_desc_tile: 64 KB of shared memory
+constexpr int kCrtTileLog = 12;                // k_desc_crt's words per prime: 80 KB of shared memory
+constexpr int kCrtThreads = 512;
+
+// roots under node P of size n
+__device__ __forceinline__ int64_t node_roots(int64_t T, int64_t P, int64_t n) {
+  const int64_t d = T - P * n;
+  return d < 0 ? 0 : (d > n ? n : d);
 }
 
-// Descent products: Y[c][r][i][P n + k] = XH[r][i][P n + k] spec[i][P][1 - c][k];
-// one thread per (i, P n + k) loads the two spectra once for all R rows.
-__global__ void k_desc_mul(const uint32_t* __restrict__ XH, const uint32_t* __restrict__ spec, int R, int64_t Tp,
-                           int logn, NttConsts C, uint32_t* __restrict__ Y) {
+// XH[r][i][P n + k]: the first L1 forward stages of x[k] = X_P[d_P - 1 - k]
+// (k < d_P, else 0) modulo q_i.  A CTA takes 2^(13 - L1) columns as k_ntt_cols
+// does; the five primes of a block of columns are neighbours in the grid, so
+// that X comes from DRAM once.
+__global__ void __launch_bounds__(kNttThreads) k_desc_cols(const uint64_t* __restrict__ X, int64_t T, int64_t Tp,
+                                                           int logn, int L1, int64_t tiles,
+                                                           const uint2* __restrict__ tw, int logN, NttConsts C,
+                                                           uint32_t* __restrict__ XH) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over kNP * T'
-  if (idx >= (int64_t)kNP * Tp) return;
-  const int i = (int)(idx / Tp);
-  const int64_t e = idx - (int64_t)i * Tp;
+  __shared__ uint32_t sm[kNttTile];
+  const int i = (int)(blockIdx.x % kNP);
+  const int64_t t = blockIdx.x / kNP;
+  const int64_t r = t / tiles, tile = t - r * tiles;
+  const int64_t P = tile >> L1, n = 1ll << logn;
+  const int cwl = kNttTileLog - L1, CW = 1 << cwl;
+  const int jlo0 = (int)(tile & ((1 << L1) - 1)) << cwl;
+  const int64_t d = node_roots(T, P, n);
+  if (d <= (n >> 1)) return;
+  const uint64_t* x = X + r * Tp + P * n + d - 1;
+  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads) {
+    const int64_t k = ((int64_t)(e >> cwl) << kNttTileLog) + jlo0 + (e & (CW - 1));
+    sm[e] = k < d ? residue64(x[-k], C, i) : 0u;
+  }
+  __syncthreads();
+  smem_stages<false, true>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return i; }, cwl);
+  uint32_t* out = XH + (r * kNP + i) * Tp + P * n + jlo0;
+  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads)
+    out[((int64_t)(e >> cwl) << kNttTileLog) + (e & (CW - 1))] = sm[e];
+}
+
+// Tile `tile` of row r modulo q_i: forward stages L1 .. logn-1 of XH (FIRST:
+// L1 = 0, straight from X), the products with both children's spectra
+// (Y_c takes the sibling 1 - c), and the inverse stages back to L1:
+//   Y[c][r][i][P n + k].
+// The rows of one tile are neighbours in the grid and share its spectra in L2.
+template <bool FIRST>
+__global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* __restrict__ X,
+                                                               const uint32_t* __restrict__ XH,
+                                                               const uint32_t* __restrict__ spec, int R, int64_t T,
+                                                               int64_t Tp, int logn, int L1, int64_t tiles,
+                                                               const uint2* __restrict__ tw, int logN, NttConsts C,
+                                                               uint32_t* __restrict__ Y) {
+  pdl_enter();
+  extern __shared__ __align__(16) uint32_t fsm[];   // child L's tile, child R's tile (logical words)
+  const int r = (int)(blockIdx.x % R);
+  const int64_t t = blockIdx.x / R;
+  const int i = (int)(t / tiles);
+  const int64_t tile = t - i * tiles, n = 1ll << logn;
+  const int64_t P = tile >> L1, at = tile << kNttTileLog;          // at = P n + boff
+  const uint32_t boff = (uint32_t)(at & (n - 1));
+  const int64_t d = node_roots(T, P, n);
+  if (d <= (n >> 1)) return;
   const uint32_t q = C.q[i], qi = C.qinv[i];
-  const int64_t P = e >> logn, k = e & ((1ll << logn) - 1);
-  const uint32_t* s = spec + (int64_t)i * 2 * Tp + (2 * P << logn) + k;
-  const uint32_t sL = sub_if(s[0], 2 * q), sR = sub_if(s[1ll << logn], 2 * q);
-  const int64_t all = (int64_t)R * kNP * Tp;
-  for (int r = 0; r < R; r++) {
-    const int64_t at = ((int64_t)r * kNP + i) * Tp + e;
-    const uint32_t x = sub_if(XH[at], 2 * q);
-    Y[at] = mont32(x, sR, q, qi);                   // child L: times R
-    Y[all + at] = mont32(x, sL, q, qi);             // child R: times L
+  auto prime = [=](int) { return i; };
+  if (FIRST) {
+    const uint64_t* x = X + (int64_t)r * Tp + at + d - 1;
+    for (int k = threadIdx.x; k < kNttTile; k += kTileThreads) fsm[sw(k)] = k < d ? residue64(x[-k], C, i) : 0u;
+  } else {
+    const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
+    for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
+      const uint4 v = src[e];
+      const int w = sw(4 * e);                      // sw(4 e + j) = w ^ j
+      fsm[w] = v.x;
+      fsm[w ^ 1] = v.y;
+      fsm[w ^ 2] = v.z;
+      fsm[w ^ 3] = v.w;
+    }
+  }
+  __syncthreads();
+  smem_stages<false>(fsm, 0, kNttTile, logn, L1, boff, tw, logN, C, prime);
+  const uint4* spL = reinterpret_cast<const uint4*>(spec + (int64_t)i * 2 * Tp + (2 * P << logn) + boff);
+  const uint4* spR = spL + (n >> 2);
+  constexpr int kOther = sw(kNttTile);              // sw(8192 + x) = kOther ^ sw(x)
+  for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
+    const uint4 a = spL[e], b = spR[e];
+    const uint32_t sl[4] = {a.x, a.y, a.z, a.w}, sr[4] = {b.x, b.y, b.z, b.w};
+    const int w = sw(4 * e);
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const uint32_t x = sub_if(fsm[w ^ j], 2 * q);
+      fsm[w ^ j] = mont32(x, sub_if(sr[j], 2 * q), q, qi);
+      fsm[kOther ^ w ^ j] = mont32(x, sub_if(sl[j], 2 * q), q, qi);
+    }
+  }
+  __syncthreads();
+  const uint2* itw = tw + ((size_t)kNP << logN);
+  smem_stages<true>(fsm, 0, kNttTile, logn, L1, boff, itw, logN, C, prime);
+  smem_stages<true>(fsm, kNttTile, kNttTile, logn, L1, boff, itw, logN, C, prime);
+  uint4* y = reinterpret_cast<uint4*>(Y + ((int64_t)r * kNP + i) * Tp + at);
+  const int64_t other = (int64_t)R * kNP * Tp / 4;
+  for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
+    const int w = sw(4 * e), v = kOther ^ w;
+    y[e] = make_uint4(fsm[w], fsm[w ^ 1], fsm[w ^ 2], fsm[w ^ 3]);
+    y[other + e] = make_uint4(fsm[v], fsm[v ^ 1], fsm[v ^ 2], fsm[v ^ 3]);
   }
 }
 
-// Descent Chinese remaindering: X'[r][(2P + c) h + m] = y_c[d_P - 1 - m], m < d_c.
-__global__ void k_desc_crt(const uint32_t* __restrict__ Y, int R, int64_t T, int64_t Tp, int logn, NttConsts C,
-                           CrtScale sc, Mod M, uint64_t* __restrict__ Xn) {
+// The last L1 inverse stages of Y[c][r], all five primes of 2^(12 - L1)
+// columns in one CTA, and their Chinese remaindering:
+//   X'[r][(2P + c) h + m] = y_c[d_P - 1 - m], m < d_c.
+__global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __restrict__ Y,
+                                                             const uint64_t* __restrict__ X, int R, int64_t T,
+                                                             int64_t Tp, int logn, int L1, int64_t tiles, CrtScale sc,
+                                                             Mod M, const uint2* __restrict__ itw, int logN,
+                                                             NttConsts C, uint64_t* __restrict__ Xn) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over R * T' (child slots)
-  if (idx >= (int64_t)R * Tp) return;
-  const int rr = (int)(idx / Tp);
-  const int64_t slot = idx - (int64_t)rr * Tp;             // (2P + c) h + m
-  const int64_t n = 1ll << logn, h = n >> 1;
-  const int64_t child = slot / h, m = slot - child * h;
-  const int64_t P = child >> 1;
-  const int c = (int)(child & 1);
-  int64_t d = T - P * n;
-  d = d < 0 ? 0 : (d > n ? n : d);
-  const int64_t dl = d < h ? d : h;
-  const int64_t dc = c ? d - dl : dl;
-  if (m >= dc) return;
-  const int64_t all = (int64_t)R * kNP * Tp;
-  const uint32_t* y = Y + c * all + (int64_t)rr * kNP * Tp + P * n + (d - 1 - m);
-  uint32_t res[kNP];
+  extern __shared__ __align__(16) uint32_t fsm[];   // [prime][row][column]
+  constexpr int W = 1 << kCrtTileLog;
+  const int64_t tile = blockIdx.x % tiles, cr = blockIdx.x / tiles;     // cr = c R + r
+  const int c = cr >= R ? 1 : 0;
+  const int64_t r = cr - (int64_t)c * R, n = 1ll << logn, h = n >> 1;
+  const int sub = logn - kCrtTileLog;               // 2^sub column blocks per transform
+  const int64_t P = tile >> sub;
+  const int blk = (int)(tile & ((1 << sub) - 1));
+  const int cwl = kCrtTileLog - L1, CW = 1 << cwl, jlo0 = blk << cwl;
+  const int64_t d = node_roots(T, P, n);
+  if (d <= h) {
+    if (c == 0)
+      for (int64_t m = (int64_t)blk * W + threadIdx.x; m < min(d, (int64_t)(blk + 1) * W); m += kCrtThreads)
+        Xn[r * Tp + P * n + m] = X[r * Tp + P * n + m];
+    return;
+  }
+  const uint32_t* y = Y + cr * kNP * Tp + P * n + jlo0;
+  for (int e = threadIdx.x; e < kNP * W; e += kCrtThreads) {
+    const int i = e >> kCrtTileLog, x = e & (W - 1);
+    fsm[e] = y[(int64_t)i * Tp + ((int64_t)(x >> cwl) << kNttTileLog) + (x & (CW - 1))];
+  }
+  __syncthreads();
+  smem_stages<true, true>(fsm, 0, kNP * W, L1, 0, 0u, itw, logN, C, [=](int x) { return x >> L1; }, cwl);
+  const int64_t dc = c ? d - h : h;
+  uint64_t* out = Xn + r * Tp + (2 * P + c) * h;
+  for (int e = threadIdx.x; e < W; e += kCrtThreads) {
+    const int64_t m = d - 1 - (((int64_t)(e >> cwl) << kNttTileLog) + jlo0 + (e & (CW - 1)));
+    if (m < 0 || m >= dc) continue;
+    uint32_t res[kNP];
 #pragma unroll
-  for (int i = 0; i < kNP; i++) res[i] = shoup32(y[(int64_t)i * Tp], sc.s[i], sc.sp[i], C.q[i]);
-  Xn[idx] = crt_to_p(res, C, M);
+    for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[i * W + e], sc.s[i], sc.sp[i], C.q[i]);
+    out[m] = crt_to_p(res, C, M);
+  }
 }
 
 // ---- general cyclic products (Newton's iteration) ----------------------------------
@@ -1797,6 +1892,11 @@ void configure_fused() {
     cudaFuncSetAttribute(k_tree_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
     cudaFuncSetAttribute(k_desc_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c3);
     cudaFuncSetAttribute(k_up_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
+    const int tile2 = (int)(sizeof(uint32_t) * 2 * kNttTile);
+    cudaFuncSetAttribute(k_desc_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
+    cudaFuncSetAttribute(k_desc_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
+    cudaFuncSetAttribute(k_desc_crt, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sizeof(uint32_t) * kNP << kCrtTileLog));
     cudaFuncSetAttribute(k_up_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(uint64_t) * 2 * kLeaf * (1 + kFastProbeMaxS)));
   });
@@ -2073,15 +2173,24 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
         done = true;
       }
       if (!done) {
-        const int64_t all = (int64_t)nr * kNP * Tp;
-        launch_k(k_desc_load, cdivu((int64_t)nr * Tp, 256), 256, 0, s, X, nr, T, Tp, logn, C, XH);
+        const int L1 = logn - kNttTileLog;
+        const int64_t tiles = nodes << L1;
+        const size_t smem = sizeof(uint32_t) * 2 * kNttTile;
+        if (L1) {
+          launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
+                   XH);
+          note_launch();
+        }
+        cudaEvent_t a = prof_mark(ctx, s);
+        launch_k(L1 ? k_desc_tile<false> : k_desc_tile<true>, (unsigned)(nr * tiles * kNP), kTileThreads, smem, s, X,
+                 XH, w.spec[l - 1], nr, T, Tp, logn, L1, tiles, tw, logN, C, Y);
         note_launch();
-        launch_ntt(ctx, XH, all >> logn, logn, logT, false, tw, itw, logN, C, s);
-        launch_k(k_desc_mul, cdivu((int64_t)kNP * Tp, 256), 256, 0, s, XH, w.spec[l - 1], nr, Tp, logn, C, Y);
-        note_launch();
-        launch_ntt(ctx, Y, (2 * all) >> logn, logn, logT, true, tw, itw, logN, C, s);
-        launch_k(k_desc_crt, cdivu((int64_t)nr * Tp, 256), 256, 0, s, Y, nr, T, Tp, logn, C, crt_scale(logn), M,
-                 Xn);
+        cudaEvent_t b2 = prof_mark(ctx, s);
+        const int64_t tx = nodes - ((T - (nodes - 1) * (1ll << logn)) <= (1ll << (logn - 1)) ? 1 : 0);
+        prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * kNttTileLog);
+        const int64_t blocks = nodes << (logn - kCrtTileLog);
+        launch_k(k_desc_crt, (unsigned)(2 * nr * blocks), kCrtThreads, sizeof(uint32_t) * kNP << kCrtTileLog, s, Y, X, nr,
+                 T, Tp, logn, L1, blocks, crt_scale(logn), M, itw, logN, C, Xn);
         note_launch();
       }
       std::swap(X, Xn);
