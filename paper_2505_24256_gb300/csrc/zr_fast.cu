@@ -102,14 +102,22 @@ __global__ void k_ntt_tables(int logN, NttConsts C, uint2* __restrict__ tw, uint
 // ones) act within columns of stride 2^13 (k_ntt_cols).
 
 // Shared-memory layout of the transform kernels: logical word x lives at
-// sw(x), its bank bits XORed with bits of its 32-word row (a permutation
-// within each row).  The register passes below touch 16 words at stride 1 or
-// 16, or 8 words at strides 1, 8, 16 or multiples of 32: a warp's accesses
-// then vary five bits of x (4..8; 0..3 and 8; 3..7; 0..2, 6 and 7; 0..3 and 7;
-// 0..4), and with this swizzle each of them, and every run of 32 consecutive
-// row-aligned words, hits 32 distinct banks (the five bank bits are independent
-// sums of the five).  It is linear over GF(2): sw(x ^ y) = sw(x) ^ sw(y).
-__host__ __device__ constexpr int sw(int x) { return x ^ ((x >> 5) & 15) ^ ((x >> 3) & 24) ^ ((x >> 4) & 16); }
+// pad(x), one word skipped per row of 32.  The words a + i 2^u of a group (a and
+// i 2^u without common bits) are then at pad(a) + pad(i 2^u): with u known at
+// compile time, at one register plus immediate offsets.  A warp's accesses in
+// the register passes below vary five bits of x, of which bits 0 .. 4 move the
+// bank by 1 .. 16 and bits 5 .. 9 by 1 .. 16 again: bits 4..8 (groups of 16 at
+// stride 1), 3..7 (of 8) and 0..4 (strides of 32 and more) hit 32 distinct banks
+// as they are, and for strides 16 and 8 the lanes take bit 9 (8 and 9) next to
+// their low bits, by a swap of the group's index bits.
+__host__ __device__ constexpr int pad(int x) { return x + (x >> 5); }
+// bytes of shared memory for `words` logical words
+__host__ __device__ constexpr size_t padded_bytes(size_t words) { return sizeof(uint32_t) * (words + (words + 31) / 32); }
+
+__device__ __forceinline__ int swap_bits(int g, int i, int j) {
+  const int t = ((g >> i) ^ (g >> j)) & 1;
+  return g ^ ((t << i) | (t << j));
+}
 
 // One pass of R <= 4 butterfly stages over groups of 2^R words held in
 // registers (a radix-2^R pass).  Forward (Cooley-Tukey) stages s .. s+R-1:
@@ -121,15 +129,17 @@ __host__ __device__ constexpr int sw(int x) { return x ^ ((x >> 5) & 15) ^ ((x >
 // block (K 2^(R-1-j) + (i >> (j+1))).  Logical word x (from off) sits at
 // transform position (boff + x) mod 2^logn; prime_of(x) gives its prime.
 // COLS: the buffer holds 2^cwl columns side by side instead (word x of
-// column c at x 2^cwl + c, no swizzle), one transform each; consecutive
+// column c at x 2^cwl + c, not padded), one transform each; consecutive
 // threads take consecutive columns.  U: the stride's logarithm when it is
 // known (the word offsets are then constants), else -1.
 //
-// The passes are bound by instruction issue: 7 per butterfly, the rest is
-// addresses, twiddle loads and shared-memory accesses, which a group of 16
-// spreads over 32 butterflies.  (13 stages as 1 + 3 + 3 + 3 + 3 took 19.5
-// instructions per butterfly, as 3 + 3 + 3 + 4 it
-// takes 16: 36 to 32 us for 720 tiles of 8192 words.)
+// The passes are bound by instructions: 7 per butterfly, the rest is addresses,
+// twiddle loads and shared-memory accesses, which a group of 16 spreads over
+// 32 butterflies.  (13 stages as 1 + 3 + 3 + 3 + 3 took 19.5 instructions per
+// butterfly, as 3 + 3 + 3 + 4 it took 16; with the products, loads and stores of
+// a descent tile 20, and 15.5 since the words lie at pad(x), not at an XOR of
+// their address, and the strides are known: step T = 2^20, S = 9: 20.5 to 18.9
+// ms; 125000: 2.59 to 2.48; T = 10^4, S = 21: 0.527 to 0.511.)
 template <bool INV, int R, int U, bool COLS, class PrimeOf>
 __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int logn, int s, uint32_t boff,
                                            const uint2* __restrict__ tw, int logN, const NttConsts& C,
@@ -140,23 +150,25 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
   const int blog = u + R;                               // log2 of the group's block
   const uint32_t pmask = (1u << logn) - 1;
   const uint32_t m = 1u << s;
-  // word i of a group sits at sw(off + a + (i << u)) = sw(off + a) ^ sw(i << u)
-  // (disjoint bits)
   int cst[NR];
 #pragma unroll
-  for (int i = 0; i < NR; i++) cst[i] = COLS ? i << (u + cwl) : sw(i << u);
+  for (int i = 0; i < NR; i++) cst[i] = COLS ? i << (u + cwl) : pad(i << u);
   for (int g0 = threadIdx.x; g0 < (len >> R); g0 += blockDim.x) {
     const int col = COLS ? (g0 & ((1 << cwl) - 1)) : 0;
-    const int g = COLS ? (g0 >> cwl) : g0;
+    int g = COLS ? (g0 >> cwl) : g0;
+    if (!COLS && (len & 1023) == 0) {            // (bank conflicts: see pad)
+      if (U == 4) g = swap_bits(g, 4, 9 - R);
+      if (U == 3 && R == 3) g = swap_bits(swap_bits(g, 3, 5), 4, 6);
+    }
     const int a = ((g >> u) << blog) + (g & ((1 << u) - 1));
     const int prime = prime_of(a);
     const uint32_t q = C.q[prime];
     const uint32_t kb = ((boff + (uint32_t)a) & pmask) >> blog;
     const uint2* __restrict__ twp = tw + ((int64_t)prime << logN);
-    const int sb = COLS ? (a << cwl) + col : sw(off + a);
+    uint32_t* __restrict__ p = sm + (COLS ? (a << cwl) + col : pad(off + a));
     uint32_t x[NR];
 #pragma unroll
-    for (int i = 0; i < NR; i++) x[i] = sm[COLS ? sb + cst[i] : sb ^ cst[i]];
+    for (int i = 0; i < NR; i++) x[i] = p[cst[i]];
 #pragma unroll
     for (int j = 0; j < R; j++) {
       // a stage's twiddles are contiguous and start at a multiple of their
@@ -182,7 +194,7 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
         if (!(i & hs)) butterfly<INV>(x[i], x[i + hs], w[INV ? (i >> (j + 1)) : (i >> (R - j))], q);
     }
 #pragma unroll
-    for (int i = 0; i < NR; i++) sm[COLS ? sb + cst[i] : sb ^ cst[i]] = x[i];
+    for (int i = 0; i < NR; i++) p[cst[i]] = x[i];
   }
 }
 
@@ -191,7 +203,9 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
 // ceil(K / 4) passes of three or four stages (K = logn - s_lo; one or two
 // stages when K < 3, 2 + 3 when K = 5), those of four on the smallest strides.
 // Callers synchronise before; the last pass is followed by a barrier.
-template <bool INV, bool COLS = false, class PrimeOf>
+// COMMON: the strides get code of their own (the kernels that take nearly all
+// of the time); else one body serves all.
+template <bool INV, bool COLS = false, bool COMMON = true, class PrimeOf>
 __device__ __forceinline__ void smem_stages(uint32_t* sm, int off, int len, int logn, int s_lo, uint32_t boff,
                                             const uint2* __restrict__ tw, int logN, const NttConsts& C,
                                             PrimeOf prime_of, int cwl = 0) {
@@ -199,18 +213,25 @@ __device__ __forceinline__ void smem_stages(uint32_t* sm, int off, int len, int 
   const int fours = K - 3 * np;                      // passes of four; negative: that many stages fewer in the widest
   auto pass = [&](int R, int s) {
     const int u = INV ? logn - 1 - s : logn - s - R;
+    constexpr bool KNOWN = COMMON && !COLS;
+#define ZR_PASS(R_, U_) radix_pass<INV, R_, KNOWN ? U_ : -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl)
     if (R == 4) {
-      if (COLS) radix_pass<INV, 4, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      else if (u == 0) radix_pass<INV, 4, 0, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      else if (u == 4) radix_pass<INV, 4, 4, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
-      else radix_pass<INV, 4, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      if (!KNOWN || u == 0) ZR_PASS(4, 0);
+      else if (u == 4) ZR_PASS(4, 4);
+      else ZR_PASS(4, 8);                            // K <= 14: no other
     } else if (R == 3) {
-      radix_pass<INV, 3, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      if (!KNOWN || u == 0) ZR_PASS(3, 0);
+      else if (u == 3) ZR_PASS(3, 3);
+      else if (u == 4) ZR_PASS(3, 4);
+      else if (u == 7) ZR_PASS(3, 7);
+      else if (u == 10) ZR_PASS(3, 10);
+      else ZR_PASS(3, -1);
     } else if (R == 2) {
-      radix_pass<INV, 2, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      ZR_PASS(2, -1);
     } else {
-      radix_pass<INV, 1, -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl);
+      ZR_PASS(1, -1);
     }
+#undef ZR_PASS
     __syncthreads();
   };
   if (K <= 0) return;
@@ -240,21 +261,21 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
                                                            int plane_log, int s_lo, const uint2* __restrict__ tw,
                                                            int logN, NttConsts C) {
   pdl_enter();
-  __shared__ __align__(16) uint32_t sm[kNttTile];
+  __shared__ __align__(16) uint32_t sm[pad(kNttTile)];
   const int64_t base = (int64_t)blockIdx.x * kNttTile;
   const int len = (int)((total - base) < kNttTile ? (total - base) : kNttTile);
   if ((len & 3) == 0) {
     const uint4* src = reinterpret_cast<const uint4*>(data + base);
     for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads) {
       const uint4 v = src[e];
-      const int at = sw(4 * e);                    // sw(4 e + j) = at ^ j
+      const int at = pad(4 * e);                    // pad(4 e + j) = at + j
       sm[at] = v.x;
-      sm[at ^ 1] = v.y;
-      sm[at ^ 2] = v.z;
-      sm[at ^ 3] = v.w;
+      sm[at + 1] = v.y;
+      sm[at + 2] = v.z;
+      sm[at + 3] = v.w;
     }
   } else {
-    for (int e = threadIdx.x; e < len; e += kNttThreads) sm[sw(e)] = data[base + e];
+    for (int e = threadIdx.x; e < len; e += kNttThreads) sm[pad(e)] = data[base + e];
   }
   __syncthreads();
   const int pb5 = (int)((base >> plane_log) % kNP);   // the tile's first plane, modulo 5
@@ -267,11 +288,11 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
   if ((len & 3) == 0) {
     uint4* dst = reinterpret_cast<uint4*>(data + base);
     for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads) {
-      const int at = sw(4 * e);
-      dst[e] = make_uint4(sm[at], sm[at ^ 1], sm[at ^ 2], sm[at ^ 3]);
+      const int at = pad(4 * e);
+      dst[e] = make_uint4(sm[at], sm[at + 1], sm[at + 2], sm[at + 3]);
     }
   } else {
-    for (int e = threadIdx.x; e < len; e += kNttThreads) data[base + e] = sm[sw(e)];
+    for (int e = threadIdx.x; e < len; e += kNttThreads) data[base + e] = sm[pad(e)];
   }
 }
 
@@ -436,32 +457,32 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   auto prime = [=](int) { return i; };
   if (FIRST) {
     const uint64_t* x = X + (int64_t)r * Tp + at + d - 1;
-    for (int k = threadIdx.x; k < kNttTile; k += kTileThreads) fsm[sw(k)] = k < d ? residue64(x[-k], C, i) : 0u;
+    for (int k = threadIdx.x; k < kNttTile; k += kTileThreads) fsm[pad(k)] = k < d ? residue64(x[-k], C, i) : 0u;
   } else {
     const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
     for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
       const uint4 v = src[e];
-      const int w = sw(4 * e);                      // sw(4 e + j) = w ^ j
+      const int w = pad(4 * e);                      // pad(4 e + j) = w + j
       fsm[w] = v.x;
-      fsm[w ^ 1] = v.y;
-      fsm[w ^ 2] = v.z;
-      fsm[w ^ 3] = v.w;
+      fsm[w + 1] = v.y;
+      fsm[w + 2] = v.z;
+      fsm[w + 3] = v.w;
     }
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, kNttTile, logn, L1, boff, tw, logN, C, prime);
   const uint4* spL = reinterpret_cast<const uint4*>(spec + (int64_t)i * 2 * Tp + (2 * P << logn) + boff);
   const uint4* spR = spL + (n >> 2);
-  constexpr int kOther = sw(kNttTile);              // sw(8192 + x) = kOther ^ sw(x)
+  constexpr int kOther = pad(kNttTile);              // pad(8192 + x) = kOther + pad(x)
   for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
     const uint4 a = spL[e], b = spR[e];
     const uint32_t sl[4] = {a.x, a.y, a.z, a.w}, sr[4] = {b.x, b.y, b.z, b.w};
-    const int w = sw(4 * e);
+    const int w = pad(4 * e);
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      const uint32_t x = sub_if(fsm[w ^ j], 2 * q);
-      fsm[w ^ j] = mont32(x, sub_if(sr[j], 2 * q), q, qi);
-      fsm[kOther ^ w ^ j] = mont32(x, sub_if(sl[j], 2 * q), q, qi);
+      const uint32_t x = sub_if(fsm[w + j], 2 * q);
+      fsm[w + j] = mont32(x, sub_if(sr[j], 2 * q), q, qi);
+      fsm[kOther + w + j] = mont32(x, sub_if(sl[j], 2 * q), q, qi);
     }
   }
   __syncthreads();
@@ -471,9 +492,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   uint4* y = reinterpret_cast<uint4*>(Y + ((int64_t)r * kNP + i) * Tp + at);
   const int64_t other = (int64_t)R * kNP * Tp / 4;
   for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
-    const int w = sw(4 * e), v = kOther ^ w;
-    y[e] = make_uint4(fsm[w], fsm[w ^ 1], fsm[w ^ 2], fsm[w ^ 3]);
-    y[other + e] = make_uint4(fsm[v], fsm[v ^ 1], fsm[v ^ 2], fsm[v ^ 3]);
+    const int w = pad(4 * e), v = kOther + w;
+    y[e] = make_uint4(fsm[w], fsm[w + 1], fsm[w + 2], fsm[w + 3]);
+    y[other + e] = make_uint4(fsm[v], fsm[v + 1], fsm[v + 2], fsm[v + 3]);
   }
 }
 
@@ -581,12 +602,12 @@ constexpr int kNewtonThreadsF = 1024;   // the single-CTA Newton kernel
 constexpr int kClusterThreadsMax = 1024; // cluster levels of 2^13 and 2^14
 
 // ntr transforms of size 2^logn at logical words off + t 2^logn of sm (the
-// swizzled layout), transform t modulo prime t mod 5; forward (CT) or
+// padded layout), transform t modulo prime t mod 5; forward (CT) or
 // inverse (GS) stages.
 template <bool INV>
 __device__ __forceinline__ void smem_ntt(uint32_t* sm, int off, int ntr, int logn, const uint2* __restrict__ tw,
                                          int logN, const NttConsts& C) {
-  smem_stages<INV>(sm, off, ntr << logn, logn, 0, 0u, tw, logN, C, [=](int x) { return (x >> logn) % kNP; });
+  smem_stages<INV, false, false>(sm, off, ntr << logn, logn, 0, 0u, tw, logN, C, [=](int x) { return (x >> logn) % kNP; });
 }
 
 // Nodes a fused CTA takes at transform size 2^logn.  One: packing several
@@ -616,7 +637,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_tree_fused(const uint64_t* __
     const uint64_t x = k < d ? below[child * h + k] : 0;
 #pragma unroll
     for (int i = 0; i < kNP; i++)
-      fsm[sw((((c * npc + a) * kNP + i) << logn) + k)] = k < d ? residue64(x, C, i) : (k == d ? 1u : 0u);
+      fsm[pad((((c * npc + a) * kNP + i) << logn) + k)] = k < d ? residue64(x, C, i) : (k == d ? 1u : 0u);
   }
   __syncthreads();
   smem_ntt<false>(fsm, 0, 2 * kNP * npc, logn, tw, logN, C);
@@ -625,13 +646,13 @@ __global__ void __launch_bounds__(kFusedThreads) k_tree_fused(const uint64_t* __
     const int a = t / kNP, i = t - a * kNP;
     const int64_t P = P0 + a;
     const uint32_t q = C.q[i];
-    const uint32_t x = fsm[sw(e)], y = fsm[sw(half + e)];
+    const uint32_t x = fsm[pad(e)], y = fsm[pad(half + e)];
     if (P < nodes) {
       uint32_t* sp = spec + (int64_t)i * 2 * Tp + (2 * P << logn) + k;
       sp[0] = x;
       sp[n] = y;
     }
-    fsm[sw(e)] = mont32(sub_if(x, 2 * q), sub_if(y, 2 * q), q, C.qinv[i]);
+    fsm[pad(e)] = mont32(sub_if(x, 2 * q), sub_if(y, 2 * q), q, C.qinv[i]);
   }
   __syncthreads();
   smem_ntt<true>(fsm, 0, npc * kNP, logn, tw + ((size_t)kNP << logN), logN, C);
@@ -643,7 +664,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_tree_fused(const uint64_t* __
     if (k >= d) continue;
     uint32_t res[kNP];
 #pragma unroll
-    for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[sw(((a * kNP + i) << logn) + k)], sc.s[i], sc.sp[i], C.q[i]);
+    for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[pad(((a * kNP + i) << logn) + k)], sc.s[i], sc.sp[i], C.q[i]);
     uint64_t x = crt_to_p(res, C, M);
     if (k == 0 && d == n) x = sub_mod(x, 1, M);
     coef[P * n + k] = x;
@@ -674,7 +695,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_desc_fused(const uint64_t* __
     d = d < 0 ? 0 : (d > n ? n : d);
     const uint64_t v = k < d ? x[P * n + d - 1 - k] : 0;
 #pragma unroll
-    for (int i = 0; i < kNP; i++) fsm[sw(((a * kNP + i) << logn) + k)] = k < d ? residue64(v, C, i) : 0u;
+    for (int i = 0; i < kNP; i++) fsm[pad(((a * kNP + i) << logn) + k)] = k < d ? residue64(v, C, i) : 0u;
   }
   __syncthreads();
   smem_ntt<false>(fsm, 0, npc * kNP, logn, tw, logN, C);
@@ -685,7 +706,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_desc_fused(const uint64_t* __
       const int64_t P = P0 + a;
       const uint32_t q = C.q[i];
       const uint32_t s = P < nodes ? spec[(int64_t)i * 2 * Tp + ((2 * P + (1 - c)) << logn) + k] : 0u;
-      fsm[sw(span + e)] = mont32(sub_if(fsm[sw(e)], 2 * q), sub_if(s, 2 * q), q, C.qinv[i]);
+      fsm[pad(span + e)] = mont32(sub_if(fsm[pad(e)], 2 * q), sub_if(s, 2 * q), q, C.qinv[i]);
     }
     __syncthreads();
     smem_ntt<true>(fsm, span, npc * kNP, logn, tw + ((size_t)kNP << logN), logN, C);
@@ -700,7 +721,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_desc_fused(const uint64_t* __
       uint32_t res[kNP];
 #pragma unroll
       for (int i = 0; i < kNP; i++)
-        res[i] = shoup32(fsm[sw(span + ((a * kNP + i) << logn) + (int)(d - 1 - m))], sc.s[i], sc.sp[i], C.q[i]);
+        res[i] = shoup32(fsm[pad(span + ((a * kNP + i) << logn) + (int)(d - 1 - m))], sc.s[i], sc.sp[i], C.q[i]);
       Xn[(int64_t)r * Tp + (2 * P + c) * h + m] = crt_to_p(res, C, M);
     }
     __syncthreads();
@@ -727,8 +748,8 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_fused(const uint64_t
       const uint64_t gv = t < k ? g[t] : 0;
 #pragma unroll
       for (int i = 0; i < kNP; i++) {
-        fsm[sw((i << logn) + t)] = t < nf ? residue64(fv, C, i) : 0u;
-        fsm[sw(bo + (i << logn) + t)] = t < k ? residue64(gv, C, i) : 0u;
+        fsm[pad((i << logn) + t)] = t < nf ? residue64(fv, C, i) : 0u;
+        fsm[pad(bo + (i << logn) + t)] = t < k ? residue64(gv, C, i) : 0u;
       }
     }
     __syncthreads();
@@ -736,7 +757,7 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_fused(const uint64_t
     for (int x = threadIdx.x; x < kNP * n; x += blockDim.x) {
       const int i = x >> logn;
       const uint32_t q = C.q[i];
-      fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(bo + x)], 2 * q), q, C.qinv[i]);
+      fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(bo + x)], 2 * q), q, C.qinv[i]);
     }
     __syncthreads();
     smem_ntt<true>(fsm, 0, kNP, logn, tw + ((size_t)kNP << logN), logN, C);
@@ -753,28 +774,28 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_fused(const uint64_t
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
       uint32_t res[kNP];
 #pragma unroll
-      for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[sw((i << logn) + k + t)], s[i], sp[i], C.q[i]);
+      for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[pad((i << logn) + k + t)], s[i], sp[i], C.q[i]);
       e[t] = crt_to_p(res, C, M);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
       const uint64_t ev = t < k ? e[t] : 0;
 #pragma unroll
-      for (int i = 0; i < kNP; i++) fsm[sw((i << logn) + t)] = t < k ? residue64(ev, C, i) : 0u;
+      for (int i = 0; i < kNP; i++) fsm[pad((i << logn) + t)] = t < k ? residue64(ev, C, i) : 0u;
     }
     __syncthreads();
     smem_ntt<false>(fsm, 0, kNP, logn, tw, logN, C);
     for (int x = threadIdx.x; x < kNP * n; x += blockDim.x) {
       const int i = x >> logn;
       const uint32_t q = C.q[i];
-      fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(bo + x)], 2 * q), q, C.qinv[i]);
+      fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(bo + x)], 2 * q), q, C.qinv[i]);
     }
     __syncthreads();
     smem_ntt<true>(fsm, 0, kNP, logn, tw + ((size_t)kNP << logN), logN, C);
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
       uint32_t res[kNP];
 #pragma unroll
-      for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[sw((i << logn) + t)], s[i], sp[i], C.q[i]);
+      for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[pad((i << logn) + t)], s[i], sp[i], C.q[i]);
       const uint64_t x = crt_to_p(res, C, M);
       g[k + t] = x ? M.p - x : 0;
     }
@@ -843,13 +864,13 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
 #pragma unroll
   for (int r = 0; r < kNewtonPer; r++) {
     const int t = threadIdx.x + r * (int)blockDim.x;
-    if (t < n) fsm[sw(2 * n + t)] = v[r];
+    if (t < n) fsm[pad(2 * n + t)] = v[r];
   }
-  for (int t = threadIdx.x; t < n; t += blockDim.x) fsm[sw(n + t)] = t < k ? residue64(rd[t], C, me) : 0u;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) fsm[pad(n + t)] = t < k ? residue64(rd[t], C, me) : 0u;
   __syncthreads();
   smem_stages<false>(fsm, n, 2 * n, logn, 0, 0u, tw, logN, C, prime);   // B and g
   for (int x = threadIdx.x; x < n; x += blockDim.x)
-    fsm[sw(n + x)] = mont32(sub_if(fsm[sw(n + x)], 2 * q), sub_if(fsm[sw(2 * n + x)], 2 * q), q, qi);
+    fsm[pad(n + x)] = mont32(sub_if(fsm[pad(n + x)], 2 * q), sub_if(fsm[pad(2 * n + x)], 2 * q), q, qi);
   __syncthreads();
   smem_stages<true>(fsm, n, n, logn, 0, 0u, itw, logN, C, prime);
   cluster_sync();                                // every CTA's B holds rd g mod its prime
@@ -861,7 +882,7 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
     if (t < k) {
       uint32_t res[kNP];
 #pragma unroll
-      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(n + t)), s[j], sp[j], C.q[j]);
+      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(n + t)), s[j], sp[j], C.q[j]);
       const uint64_t x = crt_to_p(res, C, M);
       if (me == 0) ps[t] = x;
       val = residue64(x, C, me);
@@ -870,16 +891,16 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
   }
   cluster_sync();                                // B is no longer read
   // A := f mod z^T, B := q0; their product's coefficients k .. T-1
-  for (int t = threadIdx.x; t < n; t += blockDim.x) fsm[sw(t)] = (t < T && t < nf) ? residue64(f[t], C, me) : 0u;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) fsm[pad(t)] = (t < T && t < nf) ? residue64(f[t], C, me) : 0u;
 #pragma unroll
   for (int r = 0; r < kNewtonPer; r++) {
     const int t = threadIdx.x + r * (int)blockDim.x;
-    if (t < n) fsm[sw(n + t)] = v[r];
+    if (t < n) fsm[pad(n + t)] = v[r];
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);   // A and B
   for (int x = threadIdx.x; x < n; x += blockDim.x)
-    fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(n + x)], 2 * q), q, qi);
+    fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(n + x)], 2 * q), q, qi);
   __syncthreads();
   smem_stages<true>(fsm, 0, n, logn, 0, 0u, itw, logN, C, prime);
   cluster_sync();                                // every CTA's A holds f q0 mod its prime
@@ -891,7 +912,7 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
     if (t < hi) {
       uint32_t res[kNP];
 #pragma unroll
-      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(k + t)), s[j], sp[j], C.q[j]);
+      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(k + t)), s[j], sp[j], C.q[j]);
       const uint64_t fq = crt_to_p(res, C, M), a = rd[k + t];
       val = residue64(a >= fq ? a - fq : a + (M.p - fq), C, me);
     }
@@ -901,12 +922,12 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
 #pragma unroll
   for (int r = 0; r < kNewtonPer; r++) {
     const int t = threadIdx.x + r * (int)blockDim.x;
-    if (t < n) fsm[sw(t)] = v[r];
+    if (t < n) fsm[pad(t)] = v[r];
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, n, logn, 0, 0u, tw, logN, C, prime);
   for (int x = threadIdx.x; x < n; x += blockDim.x)
-    fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(2 * n + x)], 2 * q), q, qi);
+    fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(2 * n + x)], 2 * q), q, qi);
   __syncthreads();
   smem_stages<true>(fsm, 0, n, logn, 0, 0u, itw, logN, C, prime);
   cluster_sync();                                // every CTA's A holds g r mod its prime
@@ -915,7 +936,7 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
   for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
     uint32_t res[kNP];
 #pragma unroll
-    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(t)), s[j], sp[j], C.q[j]);
+    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(t)), s[j], sp[j], C.q[j]);
     ps[k + t] = crt_to_p(res, C, M);
   }
 }
@@ -923,7 +944,7 @@ __device__ __forceinline__ void newton_cluster_divide(uint32_t* fsm, int me, con
 // k_newton_fused spread over a cluster of kNP CTAs, CTA i holding prime i's
 // transforms in its shared memory: A (f, then f g, then e_hi and g e_hi: the
 // second product takes A's place once every CTA has read it), B (g's
-// spectrum) in the swizzled layout, and g mod q_i.  Each Chinese
+// spectrum) in the padded layout, and g mod q_i.  Each Chinese
 // remaindering reads the five CTAs' residues through distributed shared
 // memory, and every CTA remainders all k coefficients, so that each has e
 // (and the new g) for its own prime without a trip through global memory;
@@ -953,7 +974,7 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
   extern __shared__ uint32_t fsm[];              // A (= C) [n] at 0, B [n] at n (logical); then g mod q
   const int me = cluster_rank();
   const int K = 1 << logK;
-  uint32_t* Gq = fsm + ((2 * K + 31) & ~31);
+  uint32_t* Gq = fsm + padded_bytes(2 * K) / sizeof(uint32_t);   // pad(2 K) for K >= 16
   const uint32_t q = C.q[me], qi = C.qinv[me];
   const uint2* __restrict__ itw = tw + ((size_t)kNP << logN);
   uint32_t peer[kNP];
@@ -1002,13 +1023,13 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
   for (int lk = ilog2_dev(K1); lk < logG; lk++) {
     const int k = 1 << lk, logn = lk + 1, n = 2 * k;
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      fsm[sw(t)] = t < nf ? residue64(f[t], C, me) : 0u;
-      fsm[sw(n + t)] = t < k ? Gq[t] : 0u;
+      fsm[pad(t)] = t < nf ? residue64(f[t], C, me) : 0u;
+      fsm[pad(n + t)] = t < k ? Gq[t] : 0u;
     }
     __syncthreads();
     smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);   // A and B
     for (int x = threadIdx.x; x < n; x += blockDim.x)
-      fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(n + x)], 2 * q), q, qi);
+      fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(n + x)], 2 * q), q, qi);
     __syncthreads();
     smem_stages<true>(fsm, 0, n, logn, 0, 0u, itw, logN, C, prime);
     uint32_t s[kNP], sp[kNP];                    // 2^32 / n mod q_j: 2^(32 - logn) mod q_j
@@ -1027,7 +1048,7 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
       if (t < k) {
         uint32_t res[kNP];
 #pragma unroll
-        for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(k + t)), s[j], sp[j], C.q[j]);
+        for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(k + t)), s[j], sp[j], C.q[j]);
         v = residue64(crt_to_p(res, C, M), C, me);
       }
       ev[r] = v;
@@ -1036,19 +1057,19 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
 #pragma unroll
     for (int r = 0; r < kNewtonPer; r++) {
       const int t = threadIdx.x + r * (int)blockDim.x;
-      if (t < n) fsm[sw(t)] = ev[r];
+      if (t < n) fsm[pad(t)] = ev[r];
     }
     __syncthreads();
     smem_stages<false>(fsm, 0, n, logn, 0, 0u, tw, logN, C, prime);
     for (int x = threadIdx.x; x < n; x += blockDim.x)
-      fsm[sw(x)] = mont32(sub_if(fsm[sw(x)], 2 * q), sub_if(fsm[sw(n + x)], 2 * q), q, qi);
+      fsm[pad(x)] = mont32(sub_if(fsm[pad(x)], 2 * q), sub_if(fsm[pad(n + x)], 2 * q), q, qi);
     __syncthreads();
     smem_stages<true>(fsm, 0, n, logn, 0, 0u, itw, logN, C, prime);
     cluster_sync();                              // every CTA's C holds g e_hi mod its prime
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
       uint32_t res[kNP];
 #pragma unroll
-      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(t)), s[j], sp[j], C.q[j]);
+      for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(t)), s[j], sp[j], C.q[j]);
       const uint64_t x = crt_to_p(res, C, M);
       const uint64_t gv = x ? M.p - x : 0;
       Gq[k + t] = residue64(gv, C, me);
@@ -1110,18 +1131,18 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_tree_cluster(const uint6
     const int64_t child = 2 * P + c;
     int64_t d = T - child * h;
     d = d < 0 ? 0 : (d > h ? h : d);
-    fsm[sw(e)] = k < d ? residue64(below[child * h + k], C, me) : (k == d ? 1u : 0u);
+    fsm[pad(e)] = k < d ? residue64(below[child * h + k], C, me) : (k == d ? 1u : 0u);
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);
   uint32_t* sp = spec ? spec + (int64_t)me * 2 * Tp + (2 * P << logn) : nullptr;
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const uint32_t x = fsm[sw(k)], y = fsm[sw(n + k)];
+    const uint32_t x = fsm[pad(k)], y = fsm[pad(n + k)];
     if (sp) {
       sp[k] = x;
       sp[n + k] = y;
     }
-    fsm[sw(k)] = mont32(sub_if(x, 2 * q), sub_if(y, 2 * q), q, qi);
+    fsm[pad(k)] = mont32(sub_if(x, 2 * q), sub_if(y, 2 * q), q, qi);
   }
   if (coef == nullptr) return;                   // the children's spectra only (every CTA alike)
   __syncthreads();
@@ -1137,7 +1158,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_tree_cluster(const uint6
   for (int k = lo + threadIdx.x; k < hi; k += blockDim.x) {
     uint32_t res[kNP];
 #pragma unroll
-    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(k)), sc.s[j], sc.sp[j], C.q[j]);
+    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(k)), sc.s[j], sc.sp[j], C.q[j]);
     uint64_t x = crt_to_p(res, C, M);
     if (k == 0 && d == n) x = sub_mod(x, 1, M);
     coef[P * n + k] = x;
@@ -1174,14 +1195,14 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_desc_cluster(const uint6
     for (int o = lo + threadIdx.x; o < hi; o += blockDim.x) Xn[(int64_t)r * Tp + P * n + o] = x[o];
     return;
   }
-  for (int k = threadIdx.x; k < n; k += blockDim.x) fsm[sw(k)] = k < d ? residue64(x[d - 1 - k], C, me) : 0u;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) fsm[pad(k)] = k < d ? residue64(x[d - 1 - k], C, me) : 0u;
   __syncthreads();
   smem_stages<false>(fsm, 0, n, logn, 0, 0u, tw, logN, C, prime);
   const uint32_t* sp = spec + (int64_t)me * 2 * Tp + (2 * P << logn);
   for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) {
     const int c = e >> logn, k = e & (n - 1);
     const uint32_t sib = sp[((1 - c) << logn) + k];       // child c times its sibling
-    fsm[sw(n + e)] = mont32(sub_if(fsm[sw(k)], 2 * q), sub_if(sib, 2 * q), q, qi);
+    fsm[pad(n + e)] = mont32(sub_if(fsm[pad(k)], 2 * q), sub_if(sib, 2 * q), q, qi);
   }
   __syncthreads();
   smem_stages<true>(fsm, n, 2 * n, logn, 0, 0u, tw + ((size_t)kNP << logN), logN, C, prime);
@@ -1198,7 +1219,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_desc_cluster(const uint6
     const int at = n + (c << logn) + (int)(d - 1 - m);
     uint32_t res[kNP];
 #pragma unroll
-    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(at)), sc.s[j], sc.sp[j], C.q[j]);
+    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(at)), sc.s[j], sc.sp[j], C.q[j]);
     Xn[(int64_t)r * Tp + (2 * P + c) * h + m] = crt_to_p(res, C, M);
   }
   cluster_sync();
@@ -1468,7 +1489,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_up_fused(const uint64_t* __re
     d = d < 0 ? 0 : (d > h ? h : d);
     const uint64_t x = k < d ? src[child * h + k] : 0;
 #pragma unroll
-    for (int i = 0; i < kNP; i++) fsm[sw((((c * npc + a) * kNP + i) << logn) + k)] = k < d ? residue64(x, C, i) : 0u;
+    for (int i = 0; i < kNP; i++) fsm[pad((((c * npc + a) * kNP + i) << logn) + k)] = k < d ? residue64(x, C, i) : 0u;
   }
   __syncthreads();
   smem_ntt<false>(fsm, 0, 2 * kNP * npc, logn, tw, logN, C);
@@ -1484,8 +1505,8 @@ __global__ void __launch_bounds__(kFusedThreads) k_up_fused(const uint64_t* __re
       sR = sub_if(sp[n], 2 * q);
     }
     const uint32_t z =
-        mont32(sub_if(fsm[sw(e)], 2 * q), sR, q, qi) + mont32(sub_if(fsm[sw(half + e)], 2 * q), sL, q, qi);
-    fsm[sw(e)] = z;                              // < 2q
+        mont32(sub_if(fsm[pad(e)], 2 * q), sR, q, qi) + mont32(sub_if(fsm[pad(half + e)], 2 * q), sL, q, qi);
+    fsm[pad(e)] = z;                              // < 2q
   }
   __syncthreads();
   smem_ntt<true>(fsm, 0, npc * kNP, logn, tw + ((size_t)kNP << logN), logN, C);
@@ -1498,7 +1519,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_up_fused(const uint64_t* __re
     if (k >= d) continue;
     uint32_t res[kNP];
 #pragma unroll
-    for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[sw(((a * kNP + i) << logn) + k)], sc.s[i], sc.sp[i], C.q[i]);
+    for (int i = 0; i < kNP; i++) res[i] = shoup32(fsm[pad(((a * kNP + i) << logn) + k)], sc.s[i], sc.sp[i], C.q[i]);
     dst[P * n + k] = crt_to_p(res, C, M);
   }
 }
@@ -1526,14 +1547,14 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_up_cluster(const uint64_
     const int64_t child = 2 * P + c;
     int64_t d = G - child * h;
     d = d < 0 ? 0 : (d > h ? h : d);
-    fsm[sw(e)] = k < d ? residue64(src[child * h + k], C, me) : 0u;
+    fsm[pad(e)] = k < d ? residue64(src[child * h + k], C, me) : 0u;
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);
   const uint32_t* sp = spec + (int64_t)me * 2 * Gp + (2 * P << logn);
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const uint32_t sL = sub_if(sp[k], 2 * q), sR = sub_if(sp[n + k], 2 * q);
-    fsm[sw(k)] = mont32(sub_if(fsm[sw(k)], 2 * q), sR, q, qi) + mont32(sub_if(fsm[sw(n + k)], 2 * q), sL, q, qi);
+    fsm[pad(k)] = mont32(sub_if(fsm[pad(k)], 2 * q), sR, q, qi) + mont32(sub_if(fsm[pad(n + k)], 2 * q), sL, q, qi);
   }
   __syncthreads();
   smem_stages<true>(fsm, 0, n, logn, 0, 0u, tw + ((size_t)kNP << logN), logN, C, prime);
@@ -1549,7 +1570,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_up_cluster(const uint64_
   for (int k = lo + threadIdx.x; k < hi; k += blockDim.x) {
     uint32_t res[kNP];
 #pragma unroll
-    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * sw(k)), sc.s[j], sc.sp[j], C.q[j]);
+    for (int j = 0; j < kNP; j++) res[j] = shoup32(ld_cluster(peer[j] + 4u * pad(k)), sc.s[j], sc.sp[j], C.q[j]);
     dst[k] = crt_to_p(res, C, M);
   }
   cluster_sync();
@@ -1835,11 +1856,11 @@ cudaError_t launch_cluster(void (*kernel)(P...), int64_t clusters, int threads, 
   return e;
 }
 
-// Shared memory of k_newton_cluster for K = 2^logK: two swizzled buffers
-// of up to K words (rounded to whole 32-word rows) and g mod q.
+// Shared memory of k_newton_cluster for K = 2^logK: two padded buffers
+// of up to K words and g mod q.
 size_t newton_cluster_smem(int logK) {
   const size_t K = (size_t)1 << logK;
-  return sizeof(uint32_t) * (((2 * K + 31) & ~(size_t)31) + K);
+  return padded_bytes(2 * K) + padded_bytes(K);
 }
 
 // Whether this device runs k_newton_cluster (a cluster of kNP CTAs with the
@@ -1883,16 +1904,16 @@ bool cluster_level(const zr_ctx* ctx, int logn, int64_t clusters) {
 void configure_fused() {
   static DeviceOnce fused_attr;
   fused_attr.run([] {
-    const int bytes = (int)(sizeof(uint32_t) * 2 * kNP * kFusedMax);
+    const int bytes = (int)padded_bytes(2 * kNP * kFusedMax);
     cudaFuncSetAttribute(k_tree_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(k_desc_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(k_up_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(k_newton_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    const int c2 = (int)(sizeof(uint32_t) * 2 << kClusterMaxLog), c3 = (int)(sizeof(uint32_t) * 3 << kClusterMaxLog);
+    const int c2 = (int)padded_bytes(2 << kClusterMaxLog), c3 = (int)padded_bytes(3 << kClusterMaxLog);
     cudaFuncSetAttribute(k_tree_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
     cudaFuncSetAttribute(k_desc_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c3);
     cudaFuncSetAttribute(k_up_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
-    const int tile2 = (int)(sizeof(uint32_t) * 2 * kNttTile);
+    const int tile2 = (int)padded_bytes(2 * kNttTile);
     cudaFuncSetAttribute(k_desc_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
     cudaFuncSetAttribute(k_desc_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
     cudaFuncSetAttribute(k_desc_crt, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1912,7 +1933,7 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
     uint32_t* sp = spec[l - 1];
     const int64_t nodes = (T + (1ll << logn) - 1) >> logn;
     if (cluster_level(ctx, logn, nodes)) {
-      const cudaError_t e = launch_cluster(k_tree_cluster, nodes, cluster_threads(ctx, logn, nodes), sizeof(uint32_t) * 2 << logn,
+      const cudaError_t e = launch_cluster(k_tree_cluster, nodes, cluster_threads(ctx, logn, nodes), padded_bytes((size_t)2 << logn),
                                            st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M, tw, logN,
                                            l <= lspec ? (uint32_t*)nullptr : sp,
                                            (l == Lt && !root) ? (uint64_t*)nullptr : coef[l]);
@@ -1921,7 +1942,7 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
     }
     if (logn <= kFusedLog) {
       const int npc = fused_npc(logn);
-      launch_k(k_tree_fused, (unsigned)((nodes + npc - 1) / npc), kFusedThreads, sizeof(uint32_t) * 2 * kNP * npc << logn, st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M,
+      launch_k(k_tree_fused, (unsigned)((nodes + npc - 1) / npc), kFusedThreads, padded_bytes((size_t)2 * kNP * npc << logn), st, coef[l - 1], T, Tp, logn, C, crt_scale(logn), M,
                                                                      tw, logN, sp, coef[l], nodes);
       note_launch();
       continue;
@@ -1958,7 +1979,7 @@ void FastRun::inverse(const uint64_t* f, int64_t nf, int64_t prec, uint64_t* g, 
   }
   if (!done) {
     logK0 = std::min(logK0, kFusedLog);
-    launch_k(k_newton_fused, 1, kNewtonThreadsF, sizeof(uint32_t) * 2 * kNP << logK0, st, f, nf, logK0, C, M, tw, logN, g,
+    launch_k(k_newton_fused, 1, kNewtonThreadsF, padded_bytes((size_t)2 * kNP << logK0), st, f, nf, logK0, C, M, tw, logN, g,
                                                                                   e);
     note_launch();
   }
@@ -2155,7 +2176,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       bool done = false;
       if (cluster_level(ctx, logn, nodes * nr)) {
         cudaEvent_t a = prof_mark(ctx, s);
-        done = launch_cluster(k_desc_cluster, nodes * nr, cluster_threads(ctx, logn, nodes * nr), sizeof(uint32_t) * 3 << logn, s, X,
+        done = launch_cluster(k_desc_cluster, nodes * nr, cluster_threads(ctx, logn, nodes * nr), padded_bytes((size_t)3 << logn), s, X,
                               T, Tp, logn, C, crt_scale(logn), M, tw, logN, w.spec[l - 1], Xn, nodes) == cudaSuccess;
         if (!done) (void)cudaGetLastError();
         cudaEvent_t b2 = prof_mark(ctx, s);
@@ -2167,7 +2188,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       if (!done && logn <= kFusedLog) {
         const int npc = fused_npc(logn);
         launch_k(k_desc_fused, (unsigned)((nodes + npc - 1) / npc * nr), kFusedThreads,
-                 sizeof(uint32_t) * 2 * kNP * npc << logn, s, X, T, Tp, logn, C, crt_scale(logn), M, tw, logN,
+                 padded_bytes((size_t)2 * kNP * npc << logn), s, X, T, Tp, logn, C, crt_scale(logn), M, tw, logN,
                  w.spec[l - 1], Xn, nodes);
         note_launch();
         done = true;
@@ -2175,7 +2196,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       if (!done) {
         const int L1 = logn - kNttTileLog;
         const int64_t tiles = nodes << L1;
-        const size_t smem = sizeof(uint32_t) * 2 * kNttTile;
+        const size_t smem = padded_bytes(2 * kNttTile);
         if (L1) {
           launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
                    XH);
@@ -2274,13 +2295,13 @@ zr_status fast_probes_enqueue(zr_ctx* ctx, int64_t G, const uint64_t* U, const u
     const int64_t nodes = (G + (1ll << logn) - 1) >> logn;
     bool done = false;
     if (cluster_level(ctx, logn, nodes * S)) {
-      done = launch_cluster(k_up_cluster, nodes * S, cluster_threads(ctx, logn, nodes * S), sizeof(uint32_t) * 2 << logn, st, Nc, G,
+      done = launch_cluster(k_up_cluster, nodes * S, cluster_threads(ctx, logn, nodes * S), padded_bytes((size_t)2 << logn), st, Nc, G,
                             Gp, logn, C, crt_scale(logn), M, tw, logN, w.spec[l - 1], Nn, nodes) == cudaSuccess;
       if (!done) (void)cudaGetLastError();
     }
     if (!done && logn <= kFusedLog) {
       const int npc = fused_npc(logn);
-      launch_k(k_up_fused, (unsigned)((nodes + npc - 1) / npc * S), kFusedThreads, sizeof(uint32_t) * 2 * kNP * npc << logn, st, Nc, G, Gp, logn, C, crt_scale(logn), M, tw, logN,
+      launch_k(k_up_fused, (unsigned)((nodes + npc - 1) / npc * S), kFusedThreads, padded_bytes((size_t)2 * kNP * npc << logn), st, Nc, G, Gp, logn, C, crt_scale(logn), M, tw, logN,
                                                                    w.spec[l - 1], Nn, nodes);
       note_launch();
       done = true;
