@@ -97,9 +97,18 @@ __global__ void k_ntt_tables(int logN, NttConsts C, uint2* __restrict__ tw, uint
 // plane is a run of transforms of size n = 2^logn.  Forward stage s (m = 2^s
 // groups of distance t = n / 2^(s+1)) pairs j and j + t of group j / 2t with
 // twiddle tw[m + group]; the inverse runs the stages in reverse order.
-// Stages with t < kNttTile / 2 act within contiguous tiles of kNttTile
-// elements (k_ntt_local); the first logn - 13 forward stages (last inverse
-// ones) act within columns of stride 2^13 (k_ntt_cols).
+// The first L1 = col_stages(logn) forward stages (last inverse ones) act within
+// columns of stride 2^(logn - L1) (k_ntt_cols), the others within contiguous
+// tiles of kNttTile elements (k_ntt_local).
+
+// 12 or 13 stages on tiles: 12 are three register passes of four, and the columns
+// have room for one stage more in as many passes unless theirs are all of four.
+// (13 on tiles throughout took 18.9 ms for a step of T = 2^20, S = 9, against
+// 18.7; 125000: 2.48, 2.47.)
+inline int col_stages(int logn) {
+  const int L = logn > kNttTileLog ? logn - kNttTileLog : 0;
+  return (L & 3) ? L + 1 : L;
+}
 
 // Shared-memory layout of the transform kernels: logical word x lives at
 // pad(x), one word skipped per row of 32.  The words a + i 2^u of a group (a and
@@ -296,9 +305,9 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
   }
 }
 
-// The first L1 = logn - 13 forward stages (the last inverse ones) of a
-// transform larger than a tile pair words 2^13 or more apart.  A CTA takes
-// 2^(13 - L1) adjacent columns of the transform's 2^L1 rows of 2^13 words:
+// The first L1 forward stages (the last inverse ones) of a transform larger than
+// a tile pair words 2^(logn - L1) or more apart.  A CTA takes 2^(13 - L1)
+// adjacent columns of the transform's 2^L1 rows of 2^(logn - L1) words:
 // stage s of the whole transform acts on each column as stage s of a
 // transform of size 2^L1, twiddles included, run as radix passes with
 // consecutive threads on consecutive columns.
@@ -306,21 +315,26 @@ template <bool INV>
 __global__ void __launch_bounds__(kNttThreads) k_ntt_cols(uint32_t* __restrict__ data, int logn, int plane_log, int L1,
                                                           const uint2* __restrict__ tw, int logN, NttConsts C) {
   pdl_enter();
-  __shared__ uint32_t sm[kNttTile];
+  __shared__ __align__(16) uint32_t sm[kNttTile];
   const int cwl = kNttTileLog - L1, CW = 1 << cwl;
-  const int64_t tbase = (int64_t)(blockIdx.x >> L1) << logn;
-  const int jlo0 = (blockIdx.x & ((1 << L1) - 1)) * CW;
-  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads) {
-    const int h = e >> cwl, c = e & (CW - 1);
-    sm[e] = data[tbase + ((int64_t)h << kNttTileLog) + jlo0 + c];
-  }
+  const int sub = logn - kNttTileLog, rl = logn - L1;   // 2^sub column blocks per transform, rows of 2^rl
+  const int64_t tbase = (int64_t)(blockIdx.x >> sub) << logn;
+  const int jlo0 = (blockIdx.x & ((1 << sub) - 1)) * CW;
+  // 2^(13 - L1) >= 8 columns: rows of whole 16-byte vectors.  (Word by word this
+  // and the descent's column kernels waited on a loop of loads: step T = 2^20 18.7
+  // against 17.8 ms, 125000 2.47 against 2.40.)
+  uint32_t* d = data + tbase + jlo0;
+#pragma unroll
+  for (int e = 4 * threadIdx.x; e < kNttTile; e += 4 * kNttThreads)
+    *reinterpret_cast<uint4*>(sm + e) =
+        *reinterpret_cast<const uint4*>(d + ((int64_t)(e >> cwl) << rl) + (e & (CW - 1)));
   __syncthreads();
   const int prime = (int)((tbase >> plane_log) % kNP);
   smem_stages<INV, true>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return prime; }, cwl);
-  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads) {
-    const int h = e >> cwl, c = e & (CW - 1);
-    data[tbase + ((int64_t)h << kNttTileLog) + jlo0 + c] = sm[e];
-  }
+#pragma unroll
+  for (int e = 4 * threadIdx.x; e < kNttTile; e += 4 * kNttThreads)
+    *reinterpret_cast<uint4*>(d + ((int64_t)(e >> cwl) << rl) + (e & (CW - 1))) =
+        *reinterpret_cast<const uint4*>(sm + e);
 }
 
 // ---- loads, products, Chinese remaindering ---------------------------------------
@@ -383,7 +397,7 @@ __global__ void k_tree_crt(const uint32_t* __restrict__ Z, int64_t T, int64_t Tp
 
 // ---- descent levels of large transforms --------------------------------------------
 //
-// A level of transforms n = 2^logn >= 2^13 (L1 = logn - 13) takes three kernels:
+// A level of transforms n = 2^logn >= 2^13 (L1 = col_stages(logn)) takes three kernels:
 // the first L1 forward stages on columns, straight from the expansions; per
 // tile of 2^13 words the other forward stages, both products and the inverse
 // stages that stay inside it; the last L1 inverse stages on columns, with the
@@ -410,25 +424,28 @@ __global__ void __launch_bounds__(kNttThreads) k_desc_cols(const uint64_t* __res
                                                            const uint2* __restrict__ tw, int logN, NttConsts C,
                                                            uint32_t* __restrict__ XH) {
   pdl_enter();
-  __shared__ uint32_t sm[kNttTile];
+  __shared__ __align__(16) uint32_t sm[kNttTile];
   const int i = (int)(blockIdx.x % kNP);
   const int64_t t = blockIdx.x / kNP;
   const int64_t r = t / tiles, tile = t - r * tiles;
-  const int64_t P = tile >> L1, n = 1ll << logn;
+  const int sub = logn - kNttTileLog, rl = logn - L1;   // 2^sub column blocks per node, rows of 2^rl
+  const int64_t P = tile >> sub, n = 1ll << logn;
   const int cwl = kNttTileLog - L1, CW = 1 << cwl;
-  const int jlo0 = (int)(tile & ((1 << L1) - 1)) << cwl;
+  const int jlo0 = (int)(tile & ((1 << sub) - 1)) << cwl;
   const int64_t d = node_roots(T, P, n);
   if (d <= (n >> 1)) return;
   const uint64_t* x = X + r * Tp + P * n + d - 1;
   for (int e = threadIdx.x; e < kNttTile; e += kNttThreads) {
-    const int64_t k = ((int64_t)(e >> cwl) << kNttTileLog) + jlo0 + (e & (CW - 1));
+    const int64_t k = ((int64_t)(e >> cwl) << rl) + jlo0 + (e & (CW - 1));
     sm[e] = k < d ? residue64(x[-k], C, i) : 0u;
   }
   __syncthreads();
   smem_stages<false, true>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return i; }, cwl);
   uint32_t* out = XH + (r * kNP + i) * Tp + P * n + jlo0;
-  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads)
-    out[((int64_t)(e >> cwl) << kNttTileLog) + (e & (CW - 1))] = sm[e];
+#pragma unroll
+  for (int e = 4 * threadIdx.x; e < kNttTile; e += 4 * kNttThreads)
+    *reinterpret_cast<uint4*>(out + ((int64_t)(e >> cwl) << rl) + (e & (CW - 1))) =
+        *reinterpret_cast<const uint4*>(sm + e);
 }
 
 // Tile `tile` of row r modulo q_i: forward stages L1 .. logn-1 of XH (FIRST:
@@ -449,7 +466,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   const int64_t t = blockIdx.x / R;
   const int i = (int)(t / tiles);
   const int64_t tile = t - i * tiles, n = 1ll << logn;
-  const int64_t P = tile >> L1, at = tile << kNttTileLog;          // at = P n + boff
+  const int64_t P = tile >> (logn - kNttTileLog), at = tile << kNttTileLog;   // at = P n + boff
   const uint32_t boff = (uint32_t)(at & (n - 1));
   const int64_t d = node_roots(T, P, n);
   if (d <= (n >> 1)) return;
@@ -512,7 +529,7 @@ __global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __r
   const int64_t tile = blockIdx.x % tiles, cr = blockIdx.x / tiles;     // cr = c R + r
   const int c = cr >= R ? 1 : 0;
   const int64_t r = cr - (int64_t)c * R, n = 1ll << logn, h = n >> 1;
-  const int sub = logn - kCrtTileLog;               // 2^sub column blocks per transform
+  const int sub = logn - kCrtTileLog, rl = logn - L1;   // 2^sub column blocks per transform, rows of 2^rl
   const int64_t P = tile >> sub;
   const int blk = (int)(tile & ((1 << sub) - 1));
   const int cwl = kCrtTileLog - L1, CW = 1 << cwl, jlo0 = blk << cwl;
@@ -524,16 +541,18 @@ __global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __r
     return;
   }
   const uint32_t* y = Y + cr * kNP * Tp + P * n + jlo0;
-  for (int e = threadIdx.x; e < kNP * W; e += kCrtThreads) {
+#pragma unroll
+  for (int e = 4 * threadIdx.x; e < kNP * W; e += 4 * kCrtThreads) {   // (2^(12 - L1) >= 8 columns)
     const int i = e >> kCrtTileLog, x = e & (W - 1);
-    fsm[e] = y[(int64_t)i * Tp + ((int64_t)(x >> cwl) << kNttTileLog) + (x & (CW - 1))];
+    *reinterpret_cast<uint4*>(fsm + e) =
+        *reinterpret_cast<const uint4*>(y + (int64_t)i * Tp + ((int64_t)(x >> cwl) << rl) + (x & (CW - 1)));
   }
   __syncthreads();
   smem_stages<true, true>(fsm, 0, kNP * W, L1, 0, 0u, itw, logN, C, [=](int x) { return x >> L1; }, cwl);
   const int64_t dc = c ? d - h : h;
   uint64_t* out = Xn + r * Tp + (2 * P + c) * h;
   for (int e = threadIdx.x; e < W; e += kCrtThreads) {
-    const int64_t m = d - 1 - (((int64_t)(e >> cwl) << kNttTileLog) + jlo0 + (e & (CW - 1)));
+    const int64_t m = d - 1 - (((int64_t)(e >> cwl) << rl) + jlo0 + (e & (CW - 1)));
     if (m < 0 || m >= dc) continue;
     uint32_t res[kNP];
 #pragma unroll
@@ -1709,9 +1728,9 @@ void launch_ntt(zr_ctx* ctx, uint32_t* data, int64_t count, int logn, int plane_
                 const uint2* itw, int logN, const NttConsts& C, cudaStream_t st) {
   if (logn <= 0 || count <= 0) return;
   const int64_t total = count << logn;
-  const int L1 = logn > kNttTileLog ? logn - kNttTileLog : 0;
+  const int L1 = col_stages(logn);
   const unsigned tiles = cdivu(total, kNttTile);
-  const unsigned cols = (unsigned)(count << L1);
+  const unsigned cols = L1 ? (unsigned)(count << (logn - kNttTileLog)) : 0;
   auto local = [&](bool inverse) {
     cudaEvent_t a = prof_mark(ctx, st);
     if (inverse)
@@ -2194,8 +2213,8 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
         done = true;
       }
       if (!done) {
-        const int L1 = logn - kNttTileLog;
-        const int64_t tiles = nodes << L1;
+        const int L1 = col_stages(logn);
+        const int64_t tiles = nodes << (logn - kNttTileLog);
         const size_t smem = padded_bytes(2 * kNttTile);
         if (L1) {
           launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
@@ -2208,7 +2227,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
         note_launch();
         cudaEvent_t b2 = prof_mark(ctx, s);
         const int64_t tx = nodes - ((T - (nodes - 1) * (1ll << logn)) <= (1ll << (logn - 1)) ? 1 : 0);
-        prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * kNttTileLog);
+        prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * (logn - L1));
         const int64_t blocks = nodes << (logn - kCrtTileLog);
         launch_k(k_desc_crt, (unsigned)(2 * nr * blocks), kCrtThreads, sizeof(uint32_t) * kNP << kCrtTileLog, s, Y, X, nr,
                  T, Tp, logn, L1, blocks, crt_scale(logn), M, itw, logN, C, Xn);
