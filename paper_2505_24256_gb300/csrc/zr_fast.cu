@@ -435,9 +435,16 @@ __global__ void __launch_bounds__(kNttThreads) k_desc_cols(const uint64_t* __res
   const int64_t d = node_roots(T, P, n);
   if (d <= (n >> 1)) return;
   const uint64_t* x = X + r * Tp + P * n + d - 1;
-  for (int e = threadIdx.x; e < kNttTile; e += kNttThreads) {
-    const int64_t k = ((int64_t)(e >> cwl) << rl) + jlo0 + (e & (CW - 1));
-    sm[e] = k < d ? residue64(x[-k], C, i) : 0u;
+  for (int e0 = threadIdx.x; e0 < kNttTile; e0 += 8 * kNttThreads) {
+    uint64_t v[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const int e = e0 + j * kNttThreads;
+      const int64_t k = ((int64_t)(e >> cwl) << rl) + jlo0 + (e & (CW - 1));
+      v[j] = k < d ? x[-k] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; j++) sm[e0 + j * kNttThreads] = residue64(v[j], C, i);
   }
   __syncthreads();
   smem_stages<false, true>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return i; }, cwl);
@@ -474,7 +481,16 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   auto prime = [=](int) { return i; };
   if (FIRST) {
     const uint64_t* x = X + (int64_t)r * Tp + at + d - 1;
-    for (int k = threadIdx.x; k < kNttTile; k += kTileThreads) fsm[pad(k)] = k < d ? residue64(x[-k], C, i) : 0u;
+    for (int k0 = threadIdx.x; k0 < kNttTile; k0 += 8 * kTileThreads) {
+      uint64_t v[8];
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        const int k = k0 + j * kTileThreads;
+        v[j] = k < d ? x[-k] : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; j++) fsm[pad(k0 + j * kTileThreads)] = residue64(v[j], C, i);
+    }
   } else {
     const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
     for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
@@ -1041,9 +1057,20 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
   __syncthreads();
   for (int lk = ilog2_dev(K1); lk < logG; lk++) {
     const int k = 1 << lk, logn = lk + 1, n = 2 * k;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      fsm[pad(t)] = t < nf ? residue64(f[t], C, me) : 0u;
-      fsm[pad(n + t)] = t < k ? Gq[t] : 0u;
+    for (int t0 = threadIdx.x; t0 < n; t0 += 4 * blockDim.x) {       // (four loads in flight)
+      uint64_t v[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int t = t0 + j * (int)blockDim.x;
+        v[j] = t < n && t < nf ? f[t] : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int t = t0 + j * (int)blockDim.x;
+        if (t >= n) break;
+        fsm[pad(t)] = residue64(v[j], C, me);
+        fsm[pad(n + t)] = t < k ? Gq[t] : 0u;
+      }
     }
     __syncthreads();
     smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);   // A and B
@@ -1145,12 +1172,18 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_tree_cluster(const uint6
   const int n = 1 << logn, h = n >> 1;
   const uint32_t q = C.q[me], qi = C.qinv[me];
   auto prime = [=](int) { return me; };
-  for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) {
-    const int c = e >> logn, k = e & (n - 1);
-    const int64_t child = 2 * P + c;
-    int64_t d = T - child * h;
-    d = d < 0 ? 0 : (d > h ? h : d);
-    fsm[pad(e)] = k < d ? residue64(below[child * h + k], C, me) : (k == d ? 1u : 0u);
+  // (four loads in flight per thread, as in k_desc_cluster)
+  for (int e0 = threadIdx.x; e0 < 2 * n; e0 += 4 * blockDim.x) {
+    uint64_t v[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const int e = e0 + j * (int)blockDim.x, k = e & (n - 1);
+      const int64_t child = 2 * P + (e >> logn);
+      const int64_t d = node_roots(T, child, h);
+      v[j] = k < d ? below[child * h + k] : (k == d ? 1u : 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) fsm[pad(e0 + j * (int)blockDim.x)] = residue64(v[j], C, me);
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);
@@ -1223,7 +1256,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_desc_cluster(const uint6
 #pragma unroll
     for (int j = 0; j < 4; j++) {
       const int k = k0 + j * (int)blockDim.x;
-      v[j] = k < d ? __ldg(x + (d - 1 - k)) : 0;
+      v[j] = k < d ? x[d - 1 - k] : 0;
     }
 #pragma unroll
     for (int j = 0; j < 4; j++) fsm[pad(k0 + j * (int)blockDim.x)] = residue64(v[j], C, me);
@@ -1236,8 +1269,8 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_desc_cluster(const uint6
     uint32_t sl[4], sr[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      sl[j] = __ldg(spL + k0 + j * (int)blockDim.x);
-      sr[j] = __ldg(spR + k0 + j * (int)blockDim.x);
+      sl[j] = spL[k0 + j * (int)blockDim.x];
+      sr[j] = spR[k0 + j * (int)blockDim.x];
     }
 #pragma unroll
     for (int j = 0; j < 4; j++) {
@@ -1585,19 +1618,33 @@ __global__ void __launch_bounds__(kClusterThreadsMax) k_up_cluster(const uint64_
   const uint32_t q = C.q[me], qi = C.qinv[me];
   auto prime = [=](int) { return me; };
   const uint64_t* src = Nprev + (int64_t)col * Gp;
-  for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) {
-    const int c = e >> logn, k = e & (n - 1);
-    const int64_t child = 2 * P + c;
-    int64_t d = G - child * h;
-    d = d < 0 ? 0 : (d > h ? h : d);
-    fsm[pad(e)] = k < d ? residue64(src[child * h + k], C, me) : 0u;
+  for (int e0 = threadIdx.x; e0 < 2 * n; e0 += 4 * blockDim.x) {   // (four loads in flight)
+    uint64_t v[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const int e = e0 + j * (int)blockDim.x, k = e & (n - 1);
+      const int64_t child = 2 * P + (e >> logn);
+      v[j] = k < node_roots(G, child, h) ? src[child * h + k] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) fsm[pad(e0 + j * (int)blockDim.x)] = residue64(v[j], C, me);
   }
   __syncthreads();
   smem_stages<false>(fsm, 0, 2 * n, logn, 0, 0u, tw, logN, C, prime);
   const uint32_t* sp = spec + (int64_t)me * 2 * Gp + (2 * P << logn);
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const uint32_t sL = sub_if(sp[k], 2 * q), sR = sub_if(sp[n + k], 2 * q);
-    fsm[pad(k)] = mont32(sub_if(fsm[pad(k)], 2 * q), sR, q, qi) + mont32(sub_if(fsm[pad(n + k)], 2 * q), sL, q, qi);
+  for (int k0 = threadIdx.x; k0 < n; k0 += 4 * blockDim.x) {
+    uint32_t sl[4], sr[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      sl[j] = sp[k0 + j * (int)blockDim.x];
+      sr[j] = sp[n + k0 + j * (int)blockDim.x];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const int k = k0 + j * (int)blockDim.x;
+      fsm[pad(k)] = mont32(sub_if(fsm[pad(k)], 2 * q), sub_if(sr[j], 2 * q), q, qi) +
+                    mont32(sub_if(fsm[pad(n + k)], 2 * q), sub_if(sl[j], 2 * q), q, qi);
+    }
   }
   __syncthreads();
   smem_stages<true>(fsm, 0, n, logn, 0, 0u, tw + ((size_t)kNP << logN), logN, C, prime);
