@@ -273,7 +273,21 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_local(uint32_t* __restrict_
   __shared__ __align__(16) uint32_t sm[pad(kNttTile)];
   const int64_t base = (int64_t)blockIdx.x * kNttTile;
   const int len = (int)((total - base) < kNttTile ? (total - base) : kNttTile);
-  if ((len & 3) == 0) {
+  if (len == kNttTile) {
+    const uint4* src = reinterpret_cast<const uint4*>(data + base);
+    constexpr int kPer = kNttTile / 4 / kNttThreads;   // all loads in flight
+    uint4 v[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; j++) v[j] = src[threadIdx.x + j * kNttThreads];
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+      const int at = pad(4 * (threadIdx.x + j * kNttThreads));      // pad(4 e + j) = at + j
+      sm[at] = v[j].x;
+      sm[at + 1] = v[j].y;
+      sm[at + 2] = v[j].z;
+      sm[at + 3] = v[j].w;
+    }
+  } else if ((len & 3) == 0) {
     const uint4* src = reinterpret_cast<const uint4*>(data + base);
     for (int e = threadIdx.x; e < (len >> 2); e += kNttThreads) {
       const uint4 v = src[e];
@@ -493,13 +507,16 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
     }
   } else {
     const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
-    for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
-      const uint4 v = src[e];
-      const int w = pad(4 * e);                      // pad(4 e + j) = w + j
-      fsm[w] = v.x;
-      fsm[w + 1] = v.y;
-      fsm[w + 2] = v.z;
-      fsm[w + 3] = v.w;
+    uint4 v[kNttTile / 4 / kTileThreads];
+#pragma unroll
+    for (int j = 0; j < kNttTile / 4 / kTileThreads; j++) v[j] = src[threadIdx.x + j * kTileThreads];
+#pragma unroll
+    for (int j = 0; j < kNttTile / 4 / kTileThreads; j++) {
+      const int w = pad(4 * (threadIdx.x + j * kTileThreads));      // pad(4 e + j) = w + j
+      fsm[w] = v[j].x;
+      fsm[w + 1] = v[j].y;
+      fsm[w + 2] = v[j].z;
+      fsm[w + 3] = v[j].w;
     }
   }
   __syncthreads();
@@ -507,15 +524,23 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   const uint4* spL = reinterpret_cast<const uint4*>(spec + (int64_t)i * 2 * Tp + (2 * P << logn) + boff);
   const uint4* spR = spL + (n >> 2);
   constexpr int kOther = pad(kNttTile);              // pad(8192 + x) = kOther + pad(x)
-  for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
-    const uint4 a = spL[e], b = spR[e];
-    const uint32_t sl[4] = {a.x, a.y, a.z, a.w}, sr[4] = {b.x, b.y, b.z, b.w};
-    const int w = pad(4 * e);
+  for (int e0 = threadIdx.x; e0 < kNttTile / 4; e0 += 2 * kTileThreads) {
+    uint4 a[2], b[2];                               // four loads in flight
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const uint32_t x = sub_if(fsm[w + j], 2 * q);
-      fsm[w + j] = mont32(x, sub_if(sr[j], 2 * q), q, qi);
-      fsm[kOther + w + j] = mont32(x, sub_if(sl[j], 2 * q), q, qi);
+    for (int t = 0; t < 2; t++) {
+      a[t] = spL[e0 + t * kTileThreads];
+      b[t] = spR[e0 + t * kTileThreads];
+    }
+#pragma unroll
+    for (int t = 0; t < 2; t++) {
+      const uint32_t sl[4] = {a[t].x, a[t].y, a[t].z, a[t].w}, sr[4] = {b[t].x, b[t].y, b[t].z, b[t].w};
+      const int w = pad(4 * (e0 + t * kTileThreads));
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const uint32_t x = sub_if(fsm[w + j], 2 * q);
+        fsm[w + j] = mont32(x, sub_if(sr[j], 2 * q), q, qi);
+        fsm[kOther + w + j] = mont32(x, sub_if(sl[j], 2 * q), q, qi);
+      }
     }
   }
   __syncthreads();
