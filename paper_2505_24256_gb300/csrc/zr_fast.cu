@@ -101,14 +101,9 @@ __global__ void k_ntt_tables(int logN, NttConsts C, uint2* __restrict__ tw, uint
 // columns of stride 2^(logn - L1) (k_ntt_cols), the others within contiguous
 // tiles of kNttTile elements (k_ntt_local).
 
-// 12 or 13 stages on tiles: 12 are three register passes of four, and the columns
-// have room for one stage more in as many passes unless theirs are all of four.
-// (13 on tiles throughout took 18.9 ms for a step of T = 2^20, S = 9, against
-// 18.7; 125000: 2.48, 2.47.)
-inline int col_stages(int logn) {
-  const int L = logn > kNttTileLog ? logn - kNttTileLog : 0;
-  return (L & 3) ? L + 1 : L;
-}
+// 12 stages on tiles: three register passes of four, on half the shared memory of
+// 13 (3 + 3 + 3 + 4; a transform of 2^13 alone has no column stages).
+inline int col_stages(int logn) { return logn > kNttTileLog ? logn - 12 : 0; }
 
 // Shared-memory layout of the transform kernels: logical word x lives at
 // pad(x), one word skipped per row of 32.  The words a + i 2^u of a group (a and
@@ -411,15 +406,21 @@ __global__ void k_tree_crt(const uint32_t* __restrict__ Z, int64_t T, int64_t Tp
 
 // ---- descent levels of large transforms --------------------------------------------
 //
-// A level of transforms n = 2^logn >= 2^13 (L1 = col_stages(logn)) takes three kernels:
+// A level of transforms n = 2^logn >= 2^13 (L1 = logn - 12) takes three kernels:
 // the first L1 forward stages on columns, straight from the expansions; per
-// tile of 2^13 words the other forward stages, both products and the inverse
+// tile of 2^12 words the other forward stages, both products and the inverse
 // stages that stay inside it; the last L1 inverse stages on columns, with the
-// Chinese remaindering.  (Loads, products and remaindering as passes of their
-// own moved 17 + 4 words of 20 bytes per coefficient, now 6 + 1.)  A node whose
-// right child holds no roots (R = 1) is copied: X_L[m] = X_P[m].
+// Chinese remaindering.  What bounds them is the transforms' instructions, not
+// memory: passes of their own for loads, products and remaindering moved 17
+// vectors of residues per level, these three 6, for 0.6 ms of 21.1 in a step of
+// T = 2^20, S = 9.  Tiles of 2^12 words in CTAs of 256 threads run 12 stages as
+// three passes, and four CTAs per SM stagger their loads, passes and barriers
+// (2^13 words, 512 threads: 16.2 ms, now 15.8; 125000: 2.23, now 2.19).  A node
+// whose right child holds no roots (R = 1) is copied: X_L[m] = X_P[m].
 
-constexpr int kTileThreads = 512;              // k_desc_tile: 64 KB of shared memory
+constexpr int kTileLog = 12;                   // k_desc_tile: two tiles of 2^12 words, 33 KB of shared memory
+constexpr int kTile = 1 << kTileLog;
+constexpr int kTileThreads = kTile / 16;       // a group of 16 each
 constexpr int kCrtTileLog = 12;                // k_desc_crt's words per prime: 80 KB of shared memory
 constexpr int kCrtThreads = 512;
 
@@ -469,14 +470,12 @@ __global__ void __launch_bounds__(kNttThreads) k_desc_cols(const uint64_t* __res
         *reinterpret_cast<const uint4*>(sm + e);
 }
 
-// Tile `tile` of row r modulo q_i: forward stages L1 .. logn-1 of XH (FIRST:
-// L1 = 0, straight from X), the products with both children's spectra
-// (Y_c takes the sibling 1 - c), and the inverse stages back to L1:
+// Tile `tile` of row r modulo q_i: forward stages L1 .. logn-1 of XH, the
+// products with both children's spectra (Y_c takes the sibling 1 - c), and the
+// inverse stages back to L1:
 //   Y[c][r][i][P n + k].
 // The rows of one tile are neighbours in the grid and share its spectra in L2.
-template <bool FIRST>
-__global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* __restrict__ X,
-                                                               const uint32_t* __restrict__ XH,
+__global__ void __launch_bounds__(kTileThreads, 4) k_desc_tile(const uint32_t* __restrict__ XH,
                                                                const uint32_t* __restrict__ spec, int R, int64_t T,
                                                                int64_t Tp, int logn, int L1, int64_t tiles,
                                                                const uint2* __restrict__ tw, int logN, NttConsts C,
@@ -487,44 +486,30 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   const int64_t t = blockIdx.x / R;
   const int i = (int)(t / tiles);
   const int64_t tile = t - i * tiles, n = 1ll << logn;
-  const int64_t P = tile >> (logn - kNttTileLog), at = tile << kNttTileLog;   // at = P n + boff
+  const int64_t P = tile >> (logn - kTileLog), at = tile << kTileLog;   // at = P n + boff
   const uint32_t boff = (uint32_t)(at & (n - 1));
   const int64_t d = node_roots(T, P, n);
   if (d <= (n >> 1)) return;
   const uint32_t q = C.q[i], qi = C.qinv[i];
   auto prime = [=](int) { return i; };
-  if (FIRST) {
-    const uint64_t* x = X + (int64_t)r * Tp + at + d - 1;
-    for (int k0 = threadIdx.x; k0 < kNttTile; k0 += 8 * kTileThreads) {
-      uint64_t v[8];
+  const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
+  uint4 v[kTile / 4 / kTileThreads];
 #pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const int k = k0 + j * kTileThreads;
-        v[j] = k < d ? x[-k] : 0;
-      }
+  for (int j = 0; j < kTile / 4 / kTileThreads; j++) v[j] = src[threadIdx.x + j * kTileThreads];
 #pragma unroll
-      for (int j = 0; j < 8; j++) fsm[pad(k0 + j * kTileThreads)] = residue64(v[j], C, i);
-    }
-  } else {
-    const uint4* src = reinterpret_cast<const uint4*>(XH + ((int64_t)r * kNP + i) * Tp + at);
-    uint4 v[kNttTile / 4 / kTileThreads];
-#pragma unroll
-    for (int j = 0; j < kNttTile / 4 / kTileThreads; j++) v[j] = src[threadIdx.x + j * kTileThreads];
-#pragma unroll
-    for (int j = 0; j < kNttTile / 4 / kTileThreads; j++) {
-      const int w = pad(4 * (threadIdx.x + j * kTileThreads));      // pad(4 e + j) = w + j
-      fsm[w] = v[j].x;
-      fsm[w + 1] = v[j].y;
-      fsm[w + 2] = v[j].z;
-      fsm[w + 3] = v[j].w;
-    }
+  for (int j = 0; j < kTile / 4 / kTileThreads; j++) {
+    const int w = pad(4 * (threadIdx.x + j * kTileThreads));      // pad(4 e + j) = w + j
+    fsm[w] = v[j].x;
+    fsm[w + 1] = v[j].y;
+    fsm[w + 2] = v[j].z;
+    fsm[w + 3] = v[j].w;
   }
   __syncthreads();
-  smem_stages<false>(fsm, 0, kNttTile, logn, L1, boff, tw, logN, C, prime);
+  smem_stages<false>(fsm, 0, kTile, logn, L1, boff, tw, logN, C, prime);
   const uint4* spL = reinterpret_cast<const uint4*>(spec + (int64_t)i * 2 * Tp + (2 * P << logn) + boff);
   const uint4* spR = spL + (n >> 2);
-  constexpr int kOther = pad(kNttTile);              // pad(8192 + x) = kOther + pad(x)
-  for (int e0 = threadIdx.x; e0 < kNttTile / 4; e0 += 2 * kTileThreads) {
+  constexpr int kOther = pad(kTile);              // pad(kTile + x) = kOther + pad(x)
+  for (int e0 = threadIdx.x; e0 < kTile / 4; e0 += 2 * kTileThreads) {
     uint4 a[2], b[2];                               // four loads in flight
 #pragma unroll
     for (int t = 0; t < 2; t++) {
@@ -545,11 +530,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_desc_tile(const uint64_t* _
   }
   __syncthreads();
   const uint2* itw = tw + ((size_t)kNP << logN);
-  smem_stages<true>(fsm, 0, kNttTile, logn, L1, boff, itw, logN, C, prime);
-  smem_stages<true>(fsm, kNttTile, kNttTile, logn, L1, boff, itw, logN, C, prime);
+  smem_stages<true>(fsm, 0, kTile, logn, L1, boff, itw, logN, C, prime);
+  smem_stages<true>(fsm, kTile, kTile, logn, L1, boff, itw, logN, C, prime);
   uint4* y = reinterpret_cast<uint4*>(Y + ((int64_t)r * kNP + i) * Tp + at);
   const int64_t other = (int64_t)R * kNP * Tp / 4;
-  for (int e = threadIdx.x; e < kNttTile / 4; e += kTileThreads) {
+  for (int e = threadIdx.x; e < kTile / 4; e += kTileThreads) {
     const int w = pad(4 * e), v = kOther + w;
     y[e] = make_uint4(fsm[w], fsm[w + 1], fsm[w + 2], fsm[w + 3]);
     y[other + e] = make_uint4(fsm[v], fsm[v + 1], fsm[v + 2], fsm[v + 3]);
@@ -2028,9 +2013,6 @@ void configure_fused() {
     cudaFuncSetAttribute(k_tree_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
     cudaFuncSetAttribute(k_desc_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c3);
     cudaFuncSetAttribute(k_up_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
-    const int tile2 = (int)padded_bytes(2 * kNttTile);
-    cudaFuncSetAttribute(k_desc_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
-    cudaFuncSetAttribute(k_desc_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile2);
     cudaFuncSetAttribute(k_desc_crt, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(uint32_t) * kNP << kCrtTileLog));
     cudaFuncSetAttribute(k_up_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2309,21 +2291,18 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
         done = true;
       }
       if (!done) {
-        const int L1 = col_stages(logn);
-        const int64_t tiles = nodes << (logn - kNttTileLog);
-        const size_t smem = padded_bytes(2 * kNttTile);
-        if (L1) {
-          launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
-                   XH);
-          note_launch();
-        }
+        const int L1 = logn - kTileLog;
+        const int64_t tiles = nodes << (logn - kNttTileLog), subs = nodes << L1;
+        launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
+                 XH);
+        note_launch();
         cudaEvent_t a = prof_mark(ctx, s);
-        launch_k(L1 ? k_desc_tile<false> : k_desc_tile<true>, (unsigned)(nr * tiles * kNP), kTileThreads, smem, s, X,
-                 XH, w.spec[l - 1], nr, T, Tp, logn, L1, tiles, tw, logN, C, Y);
+        launch_k(k_desc_tile, (unsigned)(nr * subs * kNP), kTileThreads, padded_bytes(2 * kTile), s, XH, w.spec[l - 1],
+                 nr, T, Tp, logn, L1, subs, tw, logN, C, Y);
         note_launch();
         cudaEvent_t b2 = prof_mark(ctx, s);
         const int64_t tx = nodes - ((T - (nodes - 1) * (1ll << logn)) <= (1ll << (logn - 1)) ? 1 : 0);
-        prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * (logn - L1));
+        prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * kTileLog);
         const int64_t blocks = nodes << (logn - kCrtTileLog);
         launch_k(k_desc_crt, (unsigned)(2 * nr * blocks), kCrtThreads, sizeof(uint32_t) * kNP << kCrtTileLog, s, Y, X, nr,
                  T, Tp, logn, L1, blocks, crt_scale(logn), M, itw, logN, C, Xn);
