@@ -1147,16 +1147,21 @@ __global__ void __launch_bounds__(kNewtonThreadsF) k_newton_cluster(const uint64
 // residues of a coefficient through distributed shared memory, and a last
 // barrier keeps the CTAs resident until the others are done reading.
 
-// Threads of a cluster CTA at transform size 2^logn: a quarter of the words while
-// the level's threads fit the GPU's (about 1024 per SM with these kernels'
-// registers), an eighth beyond, where whole groups of 16 words per thread cost
-// less than half-idle warps.  (Step T = 3000, S = 21: a quarter 0.292, an eighth
-// 0.306 ms; 10^4, 21: 0.550 / 0.545; 125000, 9: 2.70 / 2.64; 2^20, 9: 21.9 / 21.4.)
+// Threads of a cluster CTA at transform size 2^logn below 2^13: a quarter of the
+// words while the level's threads fit the GPU's (about 1024 per SM with these
+// kernels' registers); an eighth beyond, where whole groups of 16 words per thread
+// cost less than half-idle warps; a sixteenth, every thread a group in each pass
+// of four stages, when the CTAs fill the GPU more than twice and smaller ones
+// stagger their barriers; but no fewer than 128 (CTAs of 64 reach half the warps).
+// Step T = 2^20, S = 9: an eighth from 64 up 15.8 ms, this rule 15.6; 125000:
+// 2.19, 2.18; without the factor of two T = 10^4, S = 21 takes 0.500 ms, with it
+// 0.488.
 inline int cluster_threads(const zr_ctx* ctx, int logn, int64_t clusters) {
   if (logn >= 13) return kClusterThreadsMax;
-  const int64_t quarter = (int64_t)1 << (logn - 2);
-  const bool fits = clusters * kNP * quarter <= 1024ll * (ctx->sms ? ctx->sms : 152);
-  return (int)std::min<int64_t>(kFusedThreads, std::max<int64_t>(64, fits ? quarter : quarter / 2));
+  const int64_t room = 1024ll * (ctx->sms ? ctx->sms : 152);
+  int64_t t = std::min<int64_t>(kFusedThreads, (int64_t)1 << (logn - 2));
+  while (t > 128 && clusters * kNP * t > (t > (1 << (logn - 3)) ? room : 2 * room) && t > (1 << (logn - 4))) t /= 2;
+  return (int)t;
 }
 
 // Cluster levels go up to transforms of 2^14 (a descent CTA then holds
