@@ -351,37 +351,35 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_cols(uint32_t* __restrict__
 // Tree level l (nodes of size n = 2^l, children of size h = n/2): every child
 // c of node P as a full monic polynomial of its degree d_c (coefficients from
 // the level below, then 1, then zeros up to n), as residues:
-//   spec[i][P][c][k], plane of 2T' per prime.
+//   spec[i][P][c][k], plane of 2T' per prime; one thread per (child, k) writes
+// all five primes' residues (a thread per residue divided its index and looked up
+// its prime: 43 us a level at T = 2^20, now 11).
 __global__ void k_tree_load(const uint64_t* __restrict__ below, int64_t T, int64_t Tp, int logn, NttConsts C,
                             uint32_t* __restrict__ spec) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over kNP * 2T'
-  if (idx >= kNP * 2 * Tp) return;
-  const int i = (int)(idx / (2 * Tp));
-  const int64_t r = idx - (int64_t)i * 2 * Tp;
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over 2T'
+  if (r >= 2 * Tp) return;
   const int64_t n = 1ll << logn, h = n >> 1;
   const int64_t child = r >> logn;          // 2P + c
   const int64_t k = r & (n - 1);
   int64_t d = T - child * h;
   d = d < 0 ? 0 : (d > h ? h : d);
-  uint32_t x = 0;
-  if (k < d) x = residue64(below[child * h + k], C, i);
-  else if (k == d) x = 1;
-  spec[idx] = x;
+  const uint64_t x = k < d ? below[child * h + k] : (k == d ? 1 : 0);
+#pragma unroll
+  for (int i = 0; i < kNP; i++) spec[(int64_t)i * 2 * Tp + r] = residue64(x, C, i);
 }
 
 // Z[i][P][k] = spec_L[k] spec_R[k] (Montgomery), per prime plane of T'.
 __global__ void k_tree_mul(const uint32_t* __restrict__ spec, int64_t Tp, int logn, NttConsts C,
                            uint32_t* __restrict__ Z) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over kNP * T'
-  if (idx >= kNP * Tp) return;
-  const int i = (int)(idx / Tp);
-  const int64_t r = idx - (int64_t)i * Tp;
+  const int i = blockIdx.y;
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over T'
+  if (r >= Tp) return;
   const int64_t P = r >> logn, k = r & ((1ll << logn) - 1);
   const uint32_t q = C.q[i];
   const uint32_t* s = spec + (int64_t)i * 2 * Tp + (2 * P << logn);
-  Z[idx] = mont32(sub_if(s[k], 2 * q), sub_if(s[(1ll << logn) + k], 2 * q), q, C.qinv[i]);
+  Z[(int64_t)i * Tp + r] = mont32(sub_if(s[k], 2 * q), sub_if(s[(1ll << logn) + k], 2 * q), q, C.qinv[i]);
 }
 
 // coef[P n + k] = (L R)[k] for k < d_P, from the inverse transforms; when
@@ -592,11 +590,11 @@ __global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __r
 // A[i][k] = a[k] mod q_i for k < na, else 0 (planes of N)
 __global__ void k_cyc_load(const uint64_t* __restrict__ a, int64_t na, int logN, NttConsts C, uint32_t* __restrict__ A) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= ((int64_t)kNP << logN)) return;
-  const int i = (int)(idx >> logN);
-  const int64_t k = idx & ((1ll << logN) - 1);
-  A[idx] = k < na ? residue64(a[k], C, i) : 0;
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >> logN) return;
+  const uint64_t x = k < na ? a[k] : 0;
+#pragma unroll
+  for (int i = 0; i < kNP; i++) A[((int64_t)i << logN) + k] = residue64(x, C, i);
 }
 __global__ void k_cyc_mul(const uint32_t* __restrict__ A, const uint32_t* __restrict__ B, int logN, NttConsts C,
                           uint32_t* __restrict__ Z) {
@@ -1925,8 +1923,8 @@ struct FastRun {
   void cyc(const uint64_t* a, int64_t na, const uint64_t* b, int64_t nb, int logn, int64_t lo, int64_t cnt, bool neg,
            uint32_t* A, uint32_t* B, uint32_t* Z, uint64_t* out) {
     const int64_t all = (int64_t)kNP << logn;
-    launch_k(k_cyc_load, cdivu(all, 256), 256, 0, st, a, na, logn, C, A);
-    launch_k(k_cyc_load, cdivu(all, 256), 256, 0, st, b, nb, logn, C, B);
+    launch_k(k_cyc_load, cdivu(1ll << logn, 256), 256, 0, st, a, na, logn, C, A);
+    launch_k(k_cyc_load, cdivu(1ll << logn, 256), 256, 0, st, b, nb, logn, C, B);
     note_launches(2);
     launch_ntt(ctx, A, kNP, logn, logn, false, tw, itw, logN, C, st);
     launch_ntt(ctx, B, kNP, logn, logn, false, tw, itw, logN, C, st);
@@ -2049,10 +2047,10 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
       note_launch();
       continue;
     }
-    launch_k(k_tree_load, cdivu(kNP * 2 * Tp, 256), 256, 0, st, coef[l - 1], T, Tp, logn, C, sp);
+    launch_k(k_tree_load, cdivu(2 * Tp, 256), 256, 0, st, coef[l - 1], T, Tp, logn, C, sp);
     note_launch();
     launch_ntt(ctx, sp, (kNP * 2 * Tp) >> logn, logn, logT + 1, false, tw, itw, logN, C, st);
-    launch_k(k_tree_mul, cdivu(kNP * Tp, 256), 256, 0, st, sp, Tp, logn, C, Z);
+    launch_k(k_tree_mul, dim3(cdivu(Tp, 256), kNP), 256, 0, st, sp, Tp, logn, C, Z);
     note_launch();
     launch_ntt(ctx, Z, (kNP * Tp) >> logn, logn, logT, true, tw, itw, logN, C, st);
     launch_k(k_tree_crt, cdivu(Tp, 256), 256, 0, st, Z, T, Tp, logn, C, crt_scale(logn), M, coef[l]);
@@ -2426,7 +2424,7 @@ zr_status fast_probes_enqueue(zr_ctx* ctx, int64_t G, const uint64_t* U, const u
   const int64_t na = std::min(G, T);
   launch_k(k_rows_load, cdivu((int64_t)S << logR, 256), 256, 0, st, Nc, S, G, Gp, na, logR, C, w.A);
   note_launch();
-  launch_k(k_cyc_load, cdivu((int64_t)kNP << logR, 256), 256, 0, st, w.g, T, logR, C, w.Bg);
+  launch_k(k_cyc_load, cdivu(1ll << logR, 256), 256, 0, st, w.g, T, logR, C, w.Bg);
   note_launch();
   launch_ntt(ctx, w.A, (int64_t)S * kNP, logR, logR, false, tw, itw, logN, C, st);
   launch_ntt(ctx, w.Bg, kNP, logR, logR, false, tw, itw, logN, C, st);
