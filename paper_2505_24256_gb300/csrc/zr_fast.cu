@@ -369,17 +369,26 @@ __global__ void k_tree_load(const uint64_t* __restrict__ below, int64_t T, int64
   for (int i = 0; i < kNP; i++) spec[(int64_t)i * 2 * Tp + r] = residue64(x, C, i);
 }
 
-// Z[i][P][k] = spec_L[k] spec_R[k] (Montgomery), per prime plane of T'.
+// four products of spectra (Montgomery)
+__device__ __forceinline__ uint4 mont32x4(uint4 a, uint4 b, uint32_t q, uint32_t qi) {
+  return make_uint4(mont32(sub_if(a.x, 2 * q), sub_if(b.x, 2 * q), q, qi),
+                    mont32(sub_if(a.y, 2 * q), sub_if(b.y, 2 * q), q, qi),
+                    mont32(sub_if(a.z, 2 * q), sub_if(b.z, 2 * q), q, qi),
+                    mont32(sub_if(a.w, 2 * q), sub_if(b.w, 2 * q), q, qi));
+}
+
+// Z[i][P][k] = spec_L[k] spec_R[k], per prime plane (blockIdx.y) of T'; four k
+// per thread.
 __global__ void k_tree_mul(const uint32_t* __restrict__ spec, int64_t Tp, int logn, NttConsts C,
                            uint32_t* __restrict__ Z) {
   pdl_enter();
   const int i = blockIdx.y;
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over T'
+  const int64_t r = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);   // over T'
   if (r >= Tp) return;
   const int64_t P = r >> logn, k = r & ((1ll << logn) - 1);
-  const uint32_t q = C.q[i];
-  const uint32_t* s = spec + (int64_t)i * 2 * Tp + (2 * P << logn);
-  Z[(int64_t)i * Tp + r] = mont32(sub_if(s[k], 2 * q), sub_if(s[(1ll << logn) + k], 2 * q), q, C.qinv[i]);
+  const uint32_t* s = spec + (int64_t)i * 2 * Tp + (2 * P << logn) + k;
+  *reinterpret_cast<uint4*>(Z + (int64_t)i * Tp + r) =
+      mont32x4(*reinterpret_cast<const uint4*>(s), *reinterpret_cast<const uint4*>(s + (1ll << logn)), C.q[i], C.qinv[i]);
 }
 
 // coef[P n + k] = (L R)[k] for k < d_P, from the inverse transforms; when
@@ -596,14 +605,16 @@ __global__ void k_cyc_load(const uint64_t* __restrict__ a, int64_t na, int logN,
 #pragma unroll
   for (int i = 0; i < kNP; i++) A[((int64_t)i << logN) + k] = residue64(x, C, i);
 }
+// Z = A B per prime (blockIdx.y); four words per thread (logN >= 2)
 __global__ void k_cyc_mul(const uint32_t* __restrict__ A, const uint32_t* __restrict__ B, int logN, NttConsts C,
                           uint32_t* __restrict__ Z) {
   pdl_enter();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= ((int64_t)kNP << logN)) return;
-  const int i = (int)(idx >> logN);
-  const uint32_t q = C.q[i];
-  Z[idx] = mont32(sub_if(A[idx], 2 * q), sub_if(B[idx], 2 * q), q, C.qinv[i]);
+  const int i = blockIdx.y;
+  const int64_t k = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (k >> logN) return;
+  const int64_t at = ((int64_t)i << logN) + k;
+  *reinterpret_cast<uint4*>(Z + at) =
+      mont32x4(*reinterpret_cast<const uint4*>(A + at), *reinterpret_cast<const uint4*>(B + at), C.q[i], C.qinv[i]);
 }
 // out[t] = +-(a * b)[lo + t], t < cnt
 __global__ void k_cyc_crt(const uint32_t* __restrict__ Z, int logN, int64_t lo, int64_t cnt, int neg, NttConsts C,
@@ -1168,6 +1179,10 @@ inline int cluster_threads(const zr_ctx* ctx, int logn, int64_t clusters) {
 // nodes the tile kernels' higher occupancy wins.
 constexpr int kClusterMaxLog = 14;
 constexpr int kNewtonClusterLog = 14;
+// Where Newton's inverse leaves the cluster for transforms over the whole GPU
+// (step T = 2^20, S = 9: 14 14.80, 13 14.73, 12 14.66, 11 14.66 ms; T = 125000:
+// 1.971, 1.941, 1.948, 1.976).
+constexpr int kNewtonSeedLog = 12;
 
 // Tree level l <= kFusedLog: the children of node P as full monic
 // polynomials (modulo prime `me`) -> spectra (kept in spec for the descent)
@@ -1919,16 +1934,19 @@ struct FastRun {
   // h = rd / f mod z^T (rd: T coefficients) in one cluster, when T fits it
   // (kNewtonSchool < T <= 2^kNewtonClusterLog); false: nothing was launched
   bool quotient(const uint64_t* f, int64_t nf, const uint64_t* rd, int64_t T, uint64_t* g, uint64_t* h);
-  // out[t] = +-(a * b mod (z^N - 1))[lo + t], t < cnt; N = 2^logn
+  // out[t] = +-(a * b mod (z^N - 1))[lo + t], t < cnt; N = 2^logn.  b null: the
+  // factor whose spectrum the last call left in B (at the same logn)
   void cyc(const uint64_t* a, int64_t na, const uint64_t* b, int64_t nb, int logn, int64_t lo, int64_t cnt, bool neg,
            uint32_t* A, uint32_t* B, uint32_t* Z, uint64_t* out) {
-    const int64_t all = (int64_t)kNP << logn;
     launch_k(k_cyc_load, cdivu(1ll << logn, 256), 256, 0, st, a, na, logn, C, A);
-    launch_k(k_cyc_load, cdivu(1ll << logn, 256), 256, 0, st, b, nb, logn, C, B);
-    note_launches(2);
+    note_launch();
     launch_ntt(ctx, A, kNP, logn, logn, false, tw, itw, logN, C, st);
-    launch_ntt(ctx, B, kNP, logn, logn, false, tw, itw, logN, C, st);
-    launch_k(k_cyc_mul, cdivu(all, 256), 256, 0, st, A, B, logn, C, Z);
+    if (b) {
+      launch_k(k_cyc_load, cdivu(1ll << logn, 256), 256, 0, st, b, nb, logn, C, B);
+      note_launch();
+      launch_ntt(ctx, B, kNP, logn, logn, false, tw, itw, logN, C, st);
+    }
+    launch_k(k_cyc_mul, dim3(cdivu(1ll << logn >> 2, 256), kNP), 256, 0, st, A, B, logn, C, Z);
     note_launch();
     launch_ntt(ctx, Z, kNP, logn, logn, true, tw, itw, logN, C, st);
     launch_k(k_cyc_crt, cdivu(cnt, 256), 256, 0, st, Z, logn, lo, cnt, neg ? 1 : 0, C, crt_scale(logn), M, out);
@@ -2050,7 +2068,7 @@ void FastRun::tree(const uint64_t* v, int64_t T, int64_t Tp, int Lt, const std::
     launch_k(k_tree_load, cdivu(2 * Tp, 256), 256, 0, st, coef[l - 1], T, Tp, logn, C, sp);
     note_launch();
     launch_ntt(ctx, sp, (kNP * 2 * Tp) >> logn, logn, logT + 1, false, tw, itw, logN, C, st);
-    launch_k(k_tree_mul, dim3(cdivu(Tp, 256), kNP), 256, 0, st, sp, Tp, logn, C, Z);
+    launch_k(k_tree_mul, dim3(cdivu(Tp / 4, 256), kNP), 256, 0, st, sp, Tp, logn, C, Z);
     note_launch();
     launch_ntt(ctx, Z, (kNP * Tp) >> logn, logn, logT, true, tw, itw, logN, C, st);
     launch_k(k_tree_crt, cdivu(Tp, 256), 256, 0, st, Z, T, Tp, logn, C, crt_scale(logn), M, coef[l]);
@@ -2070,7 +2088,7 @@ bool FastRun::quotient(const uint64_t* f, int64_t nf, const uint64_t* rd, int64_
 
 void FastRun::inverse(const uint64_t* f, int64_t nf, int64_t prec, uint64_t* g, uint64_t* e, uint32_t* A,
                       uint32_t* B, uint32_t* Z) {
-  int logK0 = std::min(ilog2(prec), kNewtonClusterLog);
+  int logK0 = std::min(ilog2(prec), kNewtonSeedLog);
   bool done = false;
   if (newton_cluster_ok()) {
     done = launch_cluster(k_newton_cluster, 1, kNewtonThreadsF, newton_cluster_smem(logK0), st, f, nf, logK0, C, M,
@@ -2089,7 +2107,7 @@ void FastRun::inverse(const uint64_t* f, int64_t nf, int64_t prec, uint64_t* g, 
     // e = f g: its coefficients k .. 2k-1 (the low ones are 1, 0, ..)
     cyc(f, fn, g, k, logk2, k, k, false, A, B, Z, e);
     // g_{k..2k} = -(g e_hi mod z^k)
-    cyc(g, k, e, k, logk2, 0, k, true, A, B, Z, g + k);
+    cyc(e, k, nullptr, 0, logk2, 0, k, true, A, B, Z, g + k);   // g's spectrum is in B
   }
 }
 
