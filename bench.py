@@ -49,7 +49,7 @@ METRIC = "Zippel-step skeleton terms/s and mulmod/s vs roofline; serve p50/p99 l
 SOLVE_SOURCES = ("zr_solve.cuh", "zr_ring.cuh")
 
 
-# the sources of the transform tile kernel k_ntt_local
+# the sources of the transform kernels
 NTT_SOURCES = ("zr_fast.cu", "zr_ntt.cuh")
 
 
@@ -447,13 +447,13 @@ def probe_gen_entry(ms, S, T, G, peaks, method):
 
 
 # the profiler phases timing the fast path's transform kernels, their kernels
-FAST_KERNELS = (("desc", "k_desc_cluster"), ("ntt", "k_ntt_local"), ("psum", "k_power_sums"))
+FAST_KERNELS = (("desc", "k_desc_cluster"), ("ntt", "k_desc_tile, k_ntt_local"), ("psum", "k_power_sums"))
 
 
 def fast_roofline(ctx, peaks, workload_name, steps, step_ms):
     """Roofline entry of the O(T log^2 T) solve's dominant kernel: of the
-    descent's cluster level kernel k_desc_cluster, the transform tile kernel
-    k_ntt_local and the direct power sums kernel k_power_sums, the one with the
+    descent's cluster level kernel k_desc_cluster, the transform tile kernels
+    k_desc_tile and k_ntt_local and the direct power sums kernel k_power_sums, the one with the
     largest time in the profiled steps (each launch timed alone).  Its work
     per launch (radix-2 butterflies, n/2 per stage of each transform it runs,
     or the power sums' T^2 Shoup steps, counted by the library's profiler)

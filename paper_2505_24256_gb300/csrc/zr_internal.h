@@ -13,7 +13,7 @@
 
 // Phases of a step timed by the optional profiler (CUDA events recorded on
 // the call's stream around each phase).
-// PH_NTT times each launch of the transform tile kernel, PH_DESC each launch
+// PH_NTT times each launch of a transform tile kernel, PH_DESC each launch
 // of the descent's cluster level kernel, inside PH_FAST; both count their
 // butterflies as the phase's work.  PH_PSUM times each launch of the direct
 // power sums kernel, its T^2 Shoup steps the work.
