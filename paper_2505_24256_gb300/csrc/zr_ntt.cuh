@@ -48,17 +48,24 @@ struct CrtScale {
   uint32_t s[kNP], sp[kNP];
 };
 
+// -q modulo 2^32, opaque to the compiler: a - b q written as a + b (-q) is one
+// multiply-add, which it would otherwise turn back into a product and a difference.
+__device__ __forceinline__ uint32_t neg32(uint32_t q) {
+  uint32_t r;
+  asm("neg.s32 %0, %1;" : "=r"(r) : "r"(q));
+  return r;
+}
 // x w mod q in [0, 2q) for any 32-bit x, w < q, wp = floor(w 2^32 / q).
 __device__ __forceinline__ uint32_t shoup32(uint32_t x, uint32_t w, uint32_t wp, uint32_t q) {
-  return x * w - __umulhi(x, wp) * q;
+  return x * w + __umulhi(x, wp) * neg32(q);
 }
 // a b 2^-32 mod q in [0, q) for a b < q 2^32 (a, b < 2q suffices).
 __device__ __forceinline__ uint32_t mont32(uint32_t a, uint32_t b, uint32_t q, uint32_t qinv) {
   const uint32_t lo = a * b, hi = __umulhi(a, b);
   const uint32_t m = lo * qinv;
   const uint32_t u = __umulhi(m, q);
-  const uint32_t r = hi - u;
-  return (int32_t)r < 0 ? r + q : r;
+  const uint32_t r = hi - u;          // in (-q, q)
+  return min(r, r + q);
 }
 __device__ __forceinline__ uint32_t sub_if(uint32_t x, uint32_t b) { return min(x, x - b); }   // x - b when x >= b
 
@@ -70,7 +77,7 @@ template <bool INV>
 __device__ __forceinline__ void butterfly(uint32_t& X, uint32_t& Y, uint2 w, uint32_t q) {
   if (!INV) {
     const uint32_t x = sub_if(X, 2 * q);
-    X = Y * w.x + x - __umulhi(Y, w.y) * q;          // x + t
+    X = Y * w.x + x + __umulhi(Y, w.y) * neg32(q);   // x + t
     Y = 2 * x + 2 * q - X;                           // x - t + 2 q
   } else {
     const uint32_t x = X, y = Y;
