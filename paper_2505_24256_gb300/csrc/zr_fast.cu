@@ -131,7 +131,7 @@ __device__ __forceinline__ int swap_bits(int g, int i, int j) {
 // Inverse (Gentleman-Sande) stages s .. s-R+1: the words a + i 2^lt of one
 // block of 2^(lt+R); stage s-j pairs words 2^j apart with the twiddle of
 // block (K 2^(R-1-j) + (i >> (j+1))).  Logical word x (from off) sits at
-// transform position (boff + x) mod 2^logn; prime_of(x) gives its prime.
+// transform position (boff + (x & amask)) mod 2^logn; prime_of(x) gives its prime.
 // COLS: the buffer holds 2^cwl columns side by side instead (word x of
 // column c at x 2^cwl + c, not padded), one transform each; consecutive
 // threads take consecutive columns.  U: the stride's logarithm when it is
@@ -147,7 +147,7 @@ __device__ __forceinline__ int swap_bits(int g, int i, int j) {
 template <bool INV, int R, int U, bool COLS, class PrimeOf>
 __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int logn, int s, uint32_t boff,
                                            const uint2* __restrict__ tw, int logN, const NttConsts& C,
-                                           PrimeOf prime_of, int cwl) {
+                                           PrimeOf prime_of, int cwl, int amask) {
   constexpr int NR = 1 << R;
   const int lt = logn - 1 - s;
   const int u = U >= 0 ? U : (INV ? lt : lt - R + 1);   // log2 of the stride within a group
@@ -167,7 +167,7 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
     const int a = ((g >> u) << blog) + (g & ((1 << u) - 1));
     const int prime = prime_of(a);
     const uint32_t q = C.q[prime];
-    const uint32_t kb = ((boff + (uint32_t)a) & pmask) >> blog;
+    const uint32_t kb = ((boff + (uint32_t)(a & amask)) & pmask) >> blog;
     const uint2* __restrict__ twp = tw + ((int64_t)prime << logN);
     uint32_t* __restrict__ p = sm + (COLS ? (a << cwl) + col : pad(off + a));
     uint32_t x[NR];
@@ -212,13 +212,13 @@ __device__ __forceinline__ void radix_pass(uint32_t* sm, int off, int len, int l
 template <bool INV, bool COLS = false, bool COMMON = true, class PrimeOf>
 __device__ __forceinline__ void smem_stages(uint32_t* sm, int off, int len, int logn, int s_lo, uint32_t boff,
                                             const uint2* __restrict__ tw, int logN, const NttConsts& C,
-                                            PrimeOf prime_of, int cwl = 0) {
+                                            PrimeOf prime_of, int cwl = 0, int amask = -1) {
   const int K = logn - s_lo, np = (K + 3) >> 2;
   const int fours = K - 3 * np;                      // passes of four; negative: that many stages fewer in the widest
   auto pass = [&](int R, int s) {
     const int u = INV ? logn - 1 - s : logn - s - R;
     constexpr bool KNOWN = COMMON && !COLS;
-#define ZR_PASS(R_, U_) radix_pass<INV, R_, KNOWN ? U_ : -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl)
+#define ZR_PASS(R_, U_) radix_pass<INV, R_, KNOWN ? U_ : -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl, amask)
     if (R == 4) {
       if (!KNOWN || u == 0) ZR_PASS(4, 0);
       else if (u == 4) ZR_PASS(4, 4);
@@ -422,7 +422,9 @@ __global__ void k_tree_crt(const uint32_t* __restrict__ Z, int64_t T, int64_t Tp
 // vectors of residues per level, these three 6, for 0.6 ms of 21.1 in a step of
 // T = 2^20, S = 9.  Tiles of 2^12 words in CTAs of 256 threads run 12 stages as
 // three passes, and four CTAs per SM stagger their loads, passes and barriers
-// (2^13 words, 512 threads: 16.2 ms, now 15.8; 125000: 2.23, now 2.19).  A node
+// (2^13 words, 512 threads: 16.2 against 15.8 ms; 125000: 2.23, 2.19).  With the
+// number of stages known and both children in one pass the tile takes 42 instead
+// of 50 million warp instructions at T = 125000 (2^20: 14.5 against 14.0 ms).  A node
 // whose right child holds no roots (R = 1) is copied: X_L[m] = X_P[m].
 
 constexpr int kTileLog = 12;                   // k_desc_tile: two tiles of 2^12 words, 33 KB of shared memory
@@ -512,7 +514,8 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_desc_tile(const uint32_t* _
     fsm[w + 3] = v[j].w;
   }
   __syncthreads();
-  smem_stages<false>(fsm, 0, kTile, logn, L1, boff, tw, logN, C, prime);
+  // (the first stage as logn - 12: a known number of stages, whose passes alone are compiled)
+  smem_stages<false>(fsm, 0, kTile, logn, logn - kTileLog, boff, tw, logN, C, prime);
   const uint4* spL = reinterpret_cast<const uint4*>(spec + (int64_t)i * 2 * Tp + (2 * P << logn) + boff);
   const uint4* spR = spL + (n >> 2);
   constexpr int kOther = pad(kTile);              // pad(kTile + x) = kOther + pad(x)
@@ -537,8 +540,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_desc_tile(const uint32_t* _
   }
   __syncthreads();
   const uint2* itw = tw + ((size_t)kNP << logN);
-  smem_stages<true>(fsm, 0, kTile, logn, L1, boff, itw, logN, C, prime);
-  smem_stages<true>(fsm, kTile, kTile, logn, L1, boff, itw, logN, C, prime);
+  smem_stages<true>(fsm, 0, 2 * kTile, logn, logn - kTileLog, boff, itw, logN, C, prime, 0, kTile - 1);
   uint4* y = reinterpret_cast<uint4*>(Y + ((int64_t)r * kNP + i) * Tp + at);
   const int64_t other = (int64_t)R * kNP * Tp / 4;
   for (int e = threadIdx.x; e < kTile / 4; e += kTileThreads) {
