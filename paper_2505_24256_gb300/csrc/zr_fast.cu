@@ -217,7 +217,7 @@ __device__ __forceinline__ void smem_stages(uint32_t* sm, int off, int len, int 
   const int fours = K - 3 * np;                      // passes of four; negative: that many stages fewer in the widest
   auto pass = [&](int R, int s) {
     const int u = INV ? logn - 1 - s : logn - s - R;
-    constexpr bool KNOWN = COMMON && !COLS;
+    constexpr bool KNOWN = COMMON;
 #define ZR_PASS(R_, U_) radix_pass<INV, R_, KNOWN ? U_ : -1, COLS>(sm, off, len, logn, s, boff, tw, logN, C, prime_of, cwl, amask)
     if (R == 4) {
       if (!KNOWN || u == 0) ZR_PASS(4, 0);
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kNttThreads) k_ntt_cols(uint32_t* __restrict__
         *reinterpret_cast<const uint4*>(d + ((int64_t)(e >> cwl) << rl) + (e & (CW - 1)));
   __syncthreads();
   const int prime = (int)((tbase >> plane_log) % kNP);
-  smem_stages<INV, true>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return prime; }, cwl);
+  smem_stages<INV, true, false>(sm, 0, kNttTile, L1, 0, 0u, tw, logN, C, [=](int) { return prime; }, cwl);
 #pragma unroll
   for (int e = 4 * threadIdx.x; e < kNttTile; e += 4 * kNttThreads)
     *reinterpret_cast<uint4*>(d + ((int64_t)(e >> cwl) << rl) + (e & (CW - 1))) =
@@ -443,8 +443,9 @@ __device__ __forceinline__ int64_t node_roots(int64_t T, int64_t P, int64_t n) {
 // (k < d_P, else 0) modulo q_i.  A CTA takes 2^(13 - L1) columns as k_ntt_cols
 // does; the five primes of a block of columns are neighbours in the grid, so
 // that X comes from DRAM once.
+template <int L1>
 __global__ void __launch_bounds__(kNttThreads) k_desc_cols(const uint64_t* __restrict__ X, int64_t T, int64_t Tp,
-                                                           int logn, int L1, int64_t tiles,
+                                                           int logn, int64_t tiles,
                                                            const uint2* __restrict__ tw, int logN, NttConsts C,
                                                            uint32_t* __restrict__ XH) {
   pdl_enter();
@@ -553,9 +554,10 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_desc_tile(const uint32_t* _
 // The last L1 inverse stages of Y[c][r], all five primes of 2^(12 - L1)
 // columns in one CTA, and their Chinese remaindering:
 //   X'[r][(2P + c) h + m] = y_c[d_P - 1 - m], m < d_c.
+template <int L1>
 __global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __restrict__ Y,
                                                              const uint64_t* __restrict__ X, int R, int64_t T,
-                                                             int64_t Tp, int logn, int L1, int64_t tiles, CrtScale sc,
+                                                             int64_t Tp, int logn, int64_t tiles, CrtScale sc,
                                                              Mod M, const uint2* __restrict__ itw, int logN,
                                                              NttConsts C, uint64_t* __restrict__ Xn) {
   pdl_enter();
@@ -595,6 +597,13 @@ __global__ void __launch_bounds__(kCrtThreads, 2) k_desc_crt(const uint32_t* __r
     out[m] = crt_to_p(res, C, M);
   }
 }
+
+// The column kernels by their number of stages (1 .. 9: transforms of 2^13 to
+// 2^21), whose passes and strides are then constants (step T = 2^20, S = 9: 13.74
+// against 13.46 ms; 125000: 1.92, 1.87).
+#define ZR_BY_L1(KERNEL, L)                                                                                \
+  ((L) == 1 ? KERNEL<1> : (L) == 2 ? KERNEL<2> : (L) == 3 ? KERNEL<3> : (L) == 4 ? KERNEL<4>             \
+   : (L) == 5 ? KERNEL<5> : (L) == 6 ? KERNEL<6> : (L) == 7 ? KERNEL<7> : (L) == 8 ? KERNEL<8> : KERNEL<9>)
 
 // ---- general cyclic products (Newton's iteration) ----------------------------------
 
@@ -2048,7 +2057,8 @@ void configure_fused() {
       cudaFuncSetAttribute(ZR_BY_LOGN(k_desc_cluster, l), cudaFuncAttributeMaxDynamicSharedMemorySize, c3);
     }
     cudaFuncSetAttribute(k_up_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, c2);
-    cudaFuncSetAttribute(k_desc_crt, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    for (int l = 1; l <= 9; l++)
+      cudaFuncSetAttribute(ZR_BY_L1(k_desc_crt, l), cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(uint32_t) * kNP << kCrtTileLog));
     cudaFuncSetAttribute(k_up_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(uint64_t) * 2 * kLeaf * (1 + kFastProbeMaxS)));
@@ -2328,7 +2338,7 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
       if (!done) {
         const int L1 = logn - kTileLog;
         const int64_t tiles = nodes << (logn - kNttTileLog), subs = nodes << L1;
-        launch_k(k_desc_cols, (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, L1, tiles, tw, logN, C,
+        launch_k(ZR_BY_L1(k_desc_cols, L1), (unsigned)(nr * tiles * kNP), kNttThreads, 0, s, X, T, Tp, logn, tiles, tw, logN, C,
                  XH);
         note_launch();
         cudaEvent_t a = prof_mark(ctx, s);
@@ -2339,8 +2349,8 @@ zr_status fast_solve_enqueue(zr_ctx* ctx, int64_t T, int S, const uint64_t* v, c
         const int64_t tx = nodes - ((T - (nodes - 1) * (1ll << logn)) <= (1ll << (logn - 1)) ? 1 : 0);
         prof_add(ctx, PH_NTT, a, b2, (double)((tx * nr) << (logn - 1)) * kNP * 3 * kTileLog);
         const int64_t blocks = nodes << (logn - kCrtTileLog);
-        launch_k(k_desc_crt, (unsigned)(2 * nr * blocks), kCrtThreads, sizeof(uint32_t) * kNP << kCrtTileLog, s, Y, X, nr,
-                 T, Tp, logn, L1, blocks, crt_scale(logn), M, itw, logN, C, Xn);
+        launch_k(ZR_BY_L1(k_desc_crt, L1), (unsigned)(2 * nr * blocks), kCrtThreads, sizeof(uint32_t) * kNP << kCrtTileLog, s, Y, X, nr,
+                 T, Tp, logn, blocks, crt_scale(logn), M, itw, logN, C, Xn);
         note_launch();
       }
       std::swap(X, Xn);
