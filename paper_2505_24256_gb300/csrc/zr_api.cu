@@ -483,9 +483,10 @@ bool use_tc_probes(int64_t T, int64_t Tf, int S) {
 }  // namespace zr
 
 // Scheduling weights in multiply-accumulate equivalents (about 2e12 per
-// second on GB300).  The O(T^2) solve does S T^2 + 2.5 T^2; the fast one was
-// measured at 25 ms for T = 2^20, S = 9 and about 0.5 ms at small T, which
-// 8 (S + 6) T log2(T)^2 + 1e9 follows.  The matrix-vector evaluator does
+// second on GB300).  The O(T^2) solve does S T^2 + 2.5 T^2; the fast one took
+// 25 ms for T = 2^20, S = 9 and about 0.5 ms at small T when this was fitted,
+// which 8 (S + 6) T log2(T)^2 + 1e9 follows (13.5 and 0.2 ms now: the weight is
+// an upper estimate, so a tick ends early rather than late).  The matrix-vector evaluator does
 // S T Tf, at a quarter of the weight on the tensor cores (8e12 to 9e12 per
 // second); the transposed tree is weighted like the fast solve on max(T, Tf).
 namespace zr {
