@@ -227,7 +227,7 @@ TcMod tc_mod(const Mod& M) {
     for (int i = 0; i < e; i++) r = r * 2 % M.p;
     return (uint64_t)r;
   };
-  return TcMod{pow2(96), (uint64_t)(((unsigned __int128)pow2(110) + pow2(154)) % M.p)};
+  return TcMod{pow2(96), pow2(154)};
 }
 
 // The values of all T roots in blocks of 2^ll: rows r < R - 1 of X (stride Tp)

@@ -188,8 +188,11 @@ __device__ __forceinline__ void tc_add_chunk(uint32_t addr, TcAcc* acc) {
     }
   }
 }
-// The residue of a sum of magnitude below 2^150, carried.  c96 = 2^96 mod p,
-// bias = (2^110 + 2^154) mod p (the offsets that make the two parts positive).
+// The residue of a sum of magnitude below 2^150, carried: the words below the
+// top one are then in [0, 2^24), so that the low 96 bits are nonnegative and
+// their high word is below 2^32 < p, as reduce128 wants it for every prime.
+// c96 = 2^96 mod p, bias = 2^154 mod p (the offset that makes the top part
+// positive).
 struct TcMod {
   uint64_t c96, bias;
 };
@@ -198,8 +201,8 @@ __device__ __forceinline__ uint64_t tc_value(TcAcc a, const TcMod& K, const Mod&
   tc_carry(a);
   const int64_t x0 = (int64_t)a.w[0] + ((int64_t)a.w[1] << 24), x1 = (int64_t)a.w[2] + ((int64_t)a.w[3] << 24),
                 x2 = (int64_t)a.w[4] + ((int64_t)a.w[5] << 24);
-  const __int128 lo = (__int128)x0 + ((__int128)x1 << 48) + ((__int128)1 << 110);
-  const uint64_t r0 = reduce128((uint64_t)((unsigned __int128)lo >> 64), (uint64_t)lo, M);
+  const unsigned __int128 lo = (unsigned __int128)(uint64_t)x0 + ((unsigned __int128)(uint64_t)x1 << 48);
+  const uint64_t r0 = reduce128((uint64_t)(lo >> 64), (uint64_t)lo, M);
   const uint64_t r2 = mul_mod(reduce128(0, (uint64_t)(x2 + (1ll << 58)), M), K.c96, M);
   return sub_mod(add_mod(r0, r2, M), K.bias, M);
 }
