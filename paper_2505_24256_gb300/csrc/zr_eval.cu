@@ -786,11 +786,15 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
     launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev,
              eval_tc_ld(Tn), Tf, S, w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, w.tc.W, w.tc.Wq);
     note_launch();
-    launch_eval_tc(ctx, w.tc, w.Gdev, Tn, w.U, S, T, out, ldo, status, st);
-    if (w.tc.gsplit > 1) {
-      launch_k(k_eval_combine, dim3(cdiv(T * S, 256)), dim3(256), 0, st, T, S, w.tc.gsplit, w.Gdev, w.tc.partial, M,
-               out, ldo);
-      note_launch();
+    const int64_t slab = eval_tc_slab(Tn, T);
+    for (int64_t t0 = 0; t0 < T; t0 += slab) {
+      const int64_t Ts = std::min(slab, T - t0);
+      launch_eval_tc(ctx, w.tc, w.Gdev, Tn, w.U, S, t0, Ts, out, ldo, status, st);
+      if (w.tc.gsplit > 1) {
+        launch_k(k_eval_combine, dim3(cdiv(Ts * S, 256)), dim3(256), 0, st, Ts, S, w.tc.gsplit, w.Gdev, w.tc.partial, M,
+                 out + t0, ldo);
+        note_launch();
+      }
     }
     return cuda_err(ctx, cudaGetLastError(), "zr_zippel_probes");
   }

@@ -83,6 +83,23 @@ __global__ void __launch_bounds__(kTcRows) k_etc_pack(const uint64_t* __restrict
   for (int i = 0; i < kTcLimbs; i++) dst[i * kTcRows] = d[i];
 }
 
+// The giant steps of the next slab of rows (kEtcSlabRows): times u_g^stride,
+// the exponent of a whole slab.  A thread takes one group and kEtcNextRows rows.
+constexpr int kEtcNextRows = 16;
+__global__ void __launch_bounds__(256) k_etc_next(const uint64_t* __restrict__ U, const int64_t* __restrict__ Gdev,
+                                                  int A, int64_t ld, int64_t stride, Mod M,
+                                                  uint64_t* __restrict__ giant) {
+  pdl_enter();
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= *Gdev) return;
+  const uint64_t w = pow_mod(U[g], (uint64_t)stride, M), wq = shoup_pre(w, M);
+  const int a0 = blockIdx.y * kEtcNextRows;
+  for (int a = a0; a < A && a < a0 + kEtcNextRows; a++) {
+    uint64_t* x = giant + (int64_t)a * ld + g;
+    *x = canon(shoup_lazy(*x, w, wq, M), M);
+  }
+}
+
 // A work unit is 32 columns (a, s) (column index a S + s) and the k-steps of
 // one split; units of one split are neighbours, so that the CTAs at work read
 // the same part of A.  One persistent CTA per SM walks them through a ring of
@@ -303,9 +320,17 @@ __global__ void __launch_bounds__(kEtcThreads, 1)
 }
 
 // Scratch: the packed digits, the giant steps, the weights, the partial sums
-// of the k splits.
+// of the k splits.  The giant steps, a row of ld words per 128 probes, are held
+// for one slab of probes at a time (256 MB at most, 2^15 rows: 16384 probes or
+// more, since ld <= 2^18), so that the scratch does not grow with T; the next
+// slab's come from this one's by a product each, one for 128 S of its products.
+constexpr int64_t kEtcGiantWords = 1ll << 25, kEtcSlabRows = 1ll << 15;
 static int etc_a(int64_t T) { return (int)((T + kTcRows - 1) / kTcRows); }
 int64_t eval_tc_ld(int64_t Tn) { return (Tn + kEtcStep - 1) / kEtcStep * kEtcStep; }
+int64_t eval_tc_slab(int64_t Tn, int64_t T) {
+  const int64_t rows = std::min(kEtcSlabRows, std::max<int64_t>(1, kEtcGiantWords / eval_tc_ld(Tn)));
+  return std::min(T, rows * kTcRows);
+}
 
 // k splits: the count with the shortest longest CTA, in k-steps' time: a unit
 // costs its k-steps, three more for every chunk of eight (the drain) and eight
@@ -326,6 +351,7 @@ static int etc_split(const zr_ctx* ctx, int64_t T, int S, int64_t Tn) {
 EvalTcWs carve_eval_tc(Carver& cv, const zr_ctx* ctx, int64_t Tn, int S, int64_t T) {
   EvalTcWs w;
   const int64_t ld = eval_tc_ld(Tn);
+  T = eval_tc_slab(Tn, T);
   w.gsplit = etc_split(ctx, T, S, Tn);
   w.W = cv.take<uint64_t>((size_t)S * ld);
   w.Wq = cv.take<uint64_t>((size_t)S * ld);
@@ -335,19 +361,23 @@ EvalTcWs carve_eval_tc(Carver& cv, const zr_ctx* ctx, int64_t Tn, int S, int64_t
   return w;
 }
 
-void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t Tn, const uint64_t* U, int S, int64_t T,
-                    uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st) {
+void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t Tn, const uint64_t* U, int S, int64_t t0,
+                    int64_t T, uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st) {
   static DeviceOnce attr;
   attr.run([] { cudaFuncSetAttribute(k_eval_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEtcSmem); });
   const Mod& M = ctx->M;
   const int64_t ld = eval_tc_ld(Tn);
   const int A = etc_a(T);
   const TcMod K = tc_mod(M);
-  launch_k(k_etc_pack, dim3((unsigned)(ld / 8)), dim3(kTcRows), 0, st, U, Gdev, A, ld, M, (uint4*)w.pack, w.giant);
+  if (t0 == 0)
+    launch_k(k_etc_pack, dim3((unsigned)(ld / 8)), dim3(kTcRows), 0, st, U, Gdev, A, ld, M, (uint4*)w.pack, w.giant);
+  else
+    launch_k(k_etc_next, dim3(cdiv(ld, 256), cdiv(A, kEtcNextRows)), dim3(256), 0, st, U, Gdev, A, ld,
+             eval_tc_slab(Tn, t0), M, w.giant);
   const int tiles = (int)cdiv((int64_t)A * S, kEtcNC), sms = ctx->sms ? ctx->sms : 152;
   launch_k(k_eval_tc, dim3((unsigned)std::min(tiles * w.gsplit, sms)), dim3(kEtcThreads), kEtcSmem, st, T, S, Gdev, A,
            ld, tiles, w.gsplit, (const unsigned char*)w.pack, (const uint64_t*)w.giant, (const uint64_t*)w.W,
-           (const uint64_t*)w.Wq, M, K, out, ldo, w.partial, status);
+           (const uint64_t*)w.Wq, M, K, out + t0, ldo, w.partial, status);
   note_launches(2);
 }
 

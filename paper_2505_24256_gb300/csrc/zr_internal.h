@@ -253,10 +253,13 @@ __host__ __device__ inline int eval_tc_splits(int gsplit, int64_t G) {
   return most < 1 ? 1 : (most < gsplit ? (int)most : gsplit);
 }
 EvalTcWs carve_eval_tc(Carver& cv, const zr_ctx* ctx, int64_t Tn, int S, int64_t T);
-// out[s ldo + i] = sum_{g < *Gdev} W[g][s] U[g]^i, i < T, or the splits' partial
-// sums (gsplit > 1)
-void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t Tn, const uint64_t* U, int S, int64_t T,
-                    uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st);
+// the probes whose giant steps the scratch holds at a time (of T)
+int64_t eval_tc_slab(int64_t Tn, int64_t T);
+// out[s ldo + i] = sum_{g < *Gdev} W[g][s] U[g]^i, t0 <= i < t0 + T, or the
+// splits' partial sums (gsplit > 1): one slab of probes, called for t0 = 0 and
+// then slab by slab in order
+void launch_eval_tc(zr_ctx* ctx, const EvalTcWs& w, const int64_t* Gdev, int64_t Tn, const uint64_t* U, int S, int64_t t0,
+                    int64_t T, uint64_t* out, int64_t ldo, uint32_t* status, cudaStream_t st);
 
 // argument check of a reconstruction request (zr_recon.cu)
 zr_status check_recon_args(zr_ctx* ctx, const zr_blackbox* bb, const zr_recon_params* prm);
