@@ -185,7 +185,8 @@ typedef struct zr_vsys {
  *      call and, in a call of several systems, also T^2 (S + 5) >= 8e7
  *      (about T >= 1750 for S = 21, 3600 for S = 1); for the probes of a
  *      function of Tf terms, the transposed-tree evaluator when T, Tf >=
- *      4096 and S T Tf >= 1.5e10;
+ *      4096 and S T Tf >= 1.5e10, and for more than 2^18 terms also when
+ *      they form G >= 4096 groups with T G (S + 8) >= 1.8e9;
  *   1  always the O(T^2) method of Sec. 2.2 (Horner quotients, deferred dot
  *      products, one inverse per root);
  *   2  the O(T log^2 T) method for every T it supports.

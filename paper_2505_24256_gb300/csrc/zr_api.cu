@@ -457,6 +457,13 @@ bool use_fast_solve(const zr_ctx* ctx, int64_t T, int S, int batch_n) {
 // against 3.3 ms).
 static constexpr double kFastProbeCross = 1.5e10;
 static constexpr int64_t kFastProbeFloorT = 4096;
+// Where the tensor cores do not run (more than kTcProbeMaxTf terms) the tree's
+// other side is the integer ring kernel, about S T G 5e-10 ms + 0.15 ms for G
+// groups against the tree's 0.4 to 6 ms; they cross where T G (S + 8) is about
+// 1.8e9 (S = 1, 400000 groups: T = 4096 5.8 against 2.1, 16000 22.0 against 2.2
+// ms; 25000 groups: T = 4096 0.51 against 0.6, 16000 1.53 against 0.8 ms).  The
+// groups are counted on the device; until then Tf stands for them.
+static constexpr double kRingTreeCross = 1.8e9;
 // The tensor cores overtake the integer ring kernel near T = Tf = 2400 (S =
 // 1), 1900 (5), 1450 (11) and 1200 (21), which T min(T, Tf) (S + 4) >= 3.3e7
 // follows (T = 3000, S = 11: 0.089 against 0.132 ms; T = 1000: 0.074 against
@@ -474,7 +481,15 @@ bool use_fast_probes(const zr_ctx* ctx, int64_t T, int64_t Tf, int S) {
   if (T < 1 || Tf < 1 || T > kFastMaxT || S > kFastProbeMaxS || ctx->solve_method == 1) return false;
   if (ctx->solve_method == 2) return true;
   if (ctx->fast_min_T > 0) return T >= ctx->fast_min_T && Tf >= ctx->fast_min_T;
-  return T >= kFastProbeFloorT && Tf >= kFastProbeFloorT && (double)T * (double)Tf * (double)S >= kFastProbeCross;
+  if (T < kFastProbeFloorT || Tf < kFastProbeFloorT) return false;
+  return (double)T * (double)Tf * (double)S >= kFastProbeCross ||
+         (Tf > kTcProbeMaxTf && (double)T * (double)Tf * (double)(S + 8) >= kRingTreeCross);
+}
+bool fast_probes_by_groups(const zr_ctx* ctx, int64_t T, int64_t Tf, int S) {
+  return ctx->solve_method == 0 && ctx->fast_min_T == 0 && (double)T * (double)Tf * (double)S < kFastProbeCross;
+}
+bool use_fast_probes_groups(int64_t T, int64_t G, int S) {
+  return G >= kFastProbeFloorT && (double)T * (double)G * (double)(S + 8) >= kRingTreeCross;
 }
 bool use_tc_probes(int64_t T, int64_t Tf, int S) {
   const double col = (double)T * (double)(S + 4);

@@ -678,7 +678,9 @@ static EvalWs carve_eval(Carver& cv, const zr_ctx* ctx, int64_t Tf, int nv, int 
   w.start = cv.take<int64_t>(Tn);
   w.order = cv.take<int64_t>(Tn);
   if (method == EVAL_TC) w.tc = carve_eval_tc(cv, ctx, Tn, S, T);
-  const int64_t Tr = (method == EVAL_TC || (fast && Tn <= kFastMaxT)) ? 1 : Tn;   // kept when the tree may fall back
+  // the ring kernel's tables, kept when the tree may fall back to it
+  const bool ring = method == EVAL_RING || (fast && (Tn > kFastMaxT || fast_probes_by_groups(ctx, T, Tf, S)));
+  const int64_t Tr = ring ? Tn : 1;
   w.Wp = cv.take<uint64_t>((size_t)ring_words(S, Tr));
   w.UP = cv.take<uint64_t>((size_t)Tr * 32);
   w.UPq = cv.take<uint64_t>((size_t)Tr * 32);
@@ -748,7 +750,8 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   launch_k(k_eval_scatter, dim3(cdiv(Tf, 256)), dim3(256), 0, st, Tf, w.tg, w.tp, w.start, w.order);
   note_launches(5);
   // the transposed tree: its sizes follow the group count, read here (the
-  // matrix-vector kernel below when there are more than kFastMaxT groups)
+  // matrix-vector kernel below when there are more than kFastMaxT groups, or
+  // too few of them for the tree)
   int64_t G = 0;
   if (fast) {
     cudaError_t e = cudaMemcpyAsync(&G, w.Gdev, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
@@ -756,7 +759,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
     if (e != cudaSuccess) return cuda_err(ctx, e, "zr_zippel_probes: group count");
     if (G < 1 || G > Tn) return set_err(ctx, ZR_ERR_CUDA, "zr_zippel_probes: group count out of range");
   }
-  if (fast && G <= kFastMaxT) {
+  if (fast && G <= kFastMaxT && (!fast_probes_by_groups(ctx, T, Tf, S) || use_fast_probes_groups(T, G, S))) {
     cudaError_t e = cudaSuccess;
     const size_t wbytes = (((size_t)S * G * sizeof(uint64_t)) + 255) & ~(size_t)255;
     const size_t need = wbytes + fast_probes_ws_need(G, T, S);

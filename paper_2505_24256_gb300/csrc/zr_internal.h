@@ -218,6 +218,10 @@ double probe_work(const zr_ctx* ctx, int64_t T, int S, int64_t Tf);
 // falls back to the matrix-vector kernel when G > kFastMaxT
 constexpr int kFastProbeMaxS = 64;            // columns of the fast evaluator
 bool use_fast_probes(const zr_ctx* ctx, int64_t T, int64_t Tf, int S);
+// whether that choice waits for the number of groups G, and the choice then
+// (false: the ring kernel)
+bool fast_probes_by_groups(const zr_ctx* ctx, int64_t T, int64_t Tf, int S);
+bool use_fast_probes_groups(int64_t T, int64_t G, int S);
 // whether the matrix-vector product of the others runs on the tensor cores
 bool use_tc_probes(int64_t T, int64_t Tf, int S);
 size_t fast_probes_ws_need(int64_t G, int64_t T, int S);

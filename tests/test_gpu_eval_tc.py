@@ -46,3 +46,26 @@ def test_scratch_does_not_grow_with_the_probes(ctx, orc, T, Tf, S, offset):
         sidx = np.full(len(iidx), s)
         want = orc.zippel_probes_sampled(exps, coef, k, y, cs, z, sidx, iidx, offset=offset)
         assert np.array_equal(out[s, iidx], want)
+
+
+@pytest.mark.parametrize("G,terms,T,S,tree", [((1 << 18) + 3, 1, 4096, 1, True), (70001, 4, 4099, 2, True),
+                                              (4100, 64, 5000, 3, False)])
+def test_many_terms_take_the_tree_by_their_groups(ctx, orc, G, terms, T, S, tree):
+    """More terms than the tensor cores take: the transposed tree for enough
+    groups, the integer kernel for few."""
+    nv, k = 6, 5
+    exps = np.zeros((G * terms, nv), dtype=np.uint8)
+    code = np.arange(G)
+    for m in range(k):
+        exps[:, m] = np.repeat((code // 21**m) % 21, terms)
+    exps[:, k] = np.tile(np.arange(terms), G)
+    st = W.Stream(G, 3)
+    coef, y, cs, z = st.residues(G * terms), st.residues(k), st.residues(S), st.residues(nv)
+    ctx.profile(True)
+    out = probes(ctx, exps, coef, k, y, cs, z, T)
+    launches = ctx.profile_query("ntt")[1]
+    ctx.profile(False)
+    assert (launches > 0) == tree
+    sidx, iidx = st.below(24, S), np.concatenate([[0, T - 1], st.below(22, T)])
+    want = orc.zippel_probes_sampled(exps, coef, k, y, cs, z, sidx, iidx)
+    assert np.array_equal(out[sidx, iidx], want)
