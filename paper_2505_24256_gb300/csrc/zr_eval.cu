@@ -172,23 +172,22 @@ __global__ void k_eval_scatter(int64_t Tf, const int32_t* __restrict__ tg, const
 // s < S <= 256, handed to store(g, j, value) for the row entries j < rw,
 // column(j) the entry's column s (negative: padding, zero).
 //
-// Many or short groups: a thread per entry.  Few long ones (eight terms and
-// more on average and at most kWeightEntries entries, or 64 terms and more:
-// the early variables of a reconstruction): a block per group, its terms
-// staged 256 at a time, a warp every eighth of them, lanes the columns;
-// a thread per entry then ran through hundreds of dependent gathers (0.043 ms
-// a call on average over a reconstruction of 8000 terms against 0.012 ms).
-// With entries enough to fill the GPU it is the other way round: 0.34 against
-// 3.9 ms for 2^20 groups of nine terms.
+// Many or short groups: a thread per entry.  Few long ones (n >= 8 terms on
+// average, at most 80 n groups: the early variables of a reconstruction): a
+// block per group, its terms staged 256 at a time, a warp every eighth of them,
+// lanes the columns; a thread per entry then runs through hundreds of dependent
+// gathers.  A block's round takes about as long as 20 of those, and 1216 blocks
+// run at a time.  Whole calls, block against thread per entry, S = 1 .. 21: 32
+// terms in 1200 groups 59 against 70 us, in 10000 136 against 110; 255 in 1200
+// 100 against 158, in 16000 600 against 590; 64 in 62500 840 against 610.
 constexpr int kWeightThreads = 256;
-constexpr int64_t kWeightEntries = 1 << 16;
 template <class Column, class Store>
 __device__ __forceinline__ void group_weights(int64_t G, int64_t Tf, int S, int rw, const int64_t* __restrict__ start,
                                               const int32_t* __restrict__ cnt, const int64_t* __restrict__ order,
                                               const uint64_t* __restrict__ a, const uint8_t* __restrict__ exps, int nv,
                                               int k, const uint64_t* __restrict__ tabC, const Mod& M, Column column,
                                               Store store) {
-  if ((G * 8 <= Tf && G * rw <= kWeightEntries) || G * 64 <= Tf) {
+  if (G * 8 <= Tf && G * G <= 80 * Tf) {
     __shared__ uint64_t sa[kWeightThreads], vals[256], red[kWeightThreads / 32][32];
     __shared__ uint8_t se[kWeightThreads];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -251,6 +250,16 @@ __device__ __forceinline__ void group_weights(int64_t G, int64_t Tf, int S, int 
     }
     store(g, j, r);
   }
+}
+
+// Blocks of the kernels above for at most G groups of Tf terms: a thread per
+// entry of rw a group, or a block per group where that is the choice (at most
+// Tf / 8 groups), eight blocks an SM at most (both ways stride the grid).
+// Sized by the entries alone, a block walked up to 256 groups in sequence: 0.12
+// ms of a probe set of 16384 groups of 16 terms at S = 1.
+static unsigned weight_blocks(const zr_ctx* ctx, int64_t G, int64_t Tf, int rw) {
+  const int64_t want = std::max<int64_t>(cdiv(G * rw, kWeightThreads), std::min(G, Tf / 8));
+  return (unsigned)std::min<int64_t>(want, 8ll * (ctx->sms ? ctx->sms : 152));
 }
 
 // Where the weights of the matrix-vector kernel live: column block b
@@ -776,8 +785,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
     }
     uint64_t* W = reinterpret_cast<uint64_t*>(*fws);
     {
-      const int64_t want = cdiv(G * S, 256), cap = 8ll * (ctx->sms ? ctx->sms : 152);
-      launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev, (int64_t)0,
+      launch_k(k_eval_weights, dim3(weight_blocks(ctx, G, Tn, S)), dim3(kWeightThreads), 0, st, w.Gdev, (int64_t)0,
                Tf, S, w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, W, (uint64_t*)nullptr);
       note_launch();
     }
@@ -785,8 +793,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   }
   // the group count stays on the device: the kernels read it, sized for Tf groups
   if (method == EVAL_TC) {
-    const int64_t want = cdiv(Tn * S, 256), cap = 8ll * (ctx->sms ? ctx->sms : 152);
-    launch_k(k_eval_weights, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev,
+    launch_k(k_eval_weights, dim3(weight_blocks(ctx, Tn, Tn, S)), dim3(kWeightThreads), 0, st, w.Gdev,
              eval_tc_ld(Tn), Tf, S, w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, offset, M, w.tc.W, w.tc.Wq);
     note_launch();
     const int64_t slab = eval_tc_slab(Tn, T);
@@ -805,12 +812,11 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
   int rw = 0;
   for (int b = 0; b < L.nb; b++) rw += L.bw[b];
   {
-    const int64_t want = cdiv(Tn * rw, 256), cap = 8ll * (ctx->sms ? ctx->sms : 152);
     // squares up to the largest exponent's top bit, and u^16 for the kernel's
     // second chain
     int nsq = 5;
     while (nsq < 32 && (T + offset) >> nsq) nsq++;
-    launch_k(k_eval_finalize, dim3((unsigned)(want < cap ? want : cap)), dim3(kWeightThreads), 0, st, w.Gdev, Tn, S,
+    launch_k(k_eval_finalize, dim3(weight_blocks(ctx, Tn, Tn, rw)), dim3(kWeightThreads), 0, st, w.Gdev, Tn, S,
              w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, M, L, rw, nsq, w.Wp, w.UP, w.UPq, w.Uq);
     note_launch();
   }
