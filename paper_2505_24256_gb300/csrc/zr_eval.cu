@@ -532,23 +532,35 @@ static int ring_occupancy_t() {
   });
 }
 
+// A grid that leaves slots of the GPU empty has to be spread over the SMs: as a
+// programmatic dependent launch its CTAs come in while the kernel before it
+// drains, several to the first SMs that have room (250000 groups, T = 64, S = 4
+// / 21: 1213 / 1603 us against 593 / 745).  Short ranges of groups are launched
+// early all the same, 3 us less of 50 to 60 (at most 2^17 terms times columns;
+// the sides cross between 2^14 and 2^17, the later the more terms a group has).
+constexpr int64_t kRingSpread = 1 << 17;
 template <int CG, int G>
-static void launch_ring_t(int64_t T, int S, int s0, int offset, const int64_t* Gdev, int64_t NG, int gsplit,
+static void launch_ring_t(int sms, int64_t T, int S, int s0, int offset, const int64_t* Gdev, int64_t NG, int gsplit,
                           const uint64_t* UP,
                           const uint64_t* UPq, const uint64_t* U, const uint64_t* Uq, const uint64_t* Wb,
                           const Mod& M, uint64_t* out, int64_t ldo, uint64_t* partial, uint32_t* status,
                           cudaStream_t st) {
   using C = EvalRingCfg<CG, G>;
-  ring_occupancy_t<CG, G>();   // also sets the shared-memory attribute
+  const int occ = ring_occupancy_t<CG, G>();   // also sets the shared-memory attribute
+  const int SC = S - s0 < G * CG ? S - s0 : G * CG;   // columns of this launch
   dim3 grid(cdiv(T, C::TI), gsplit);
-  launch_k(k_eval_ring<CG, G>, grid, dim3(C::NT), C::SMEM, st, T, S, s0, offset, Gdev, NG, gsplit, UP, UPq, U, Uq, Wb,
-           M, out, ldo, partial, status);
+  if ((int64_t)grid.x * gsplit < (int64_t)sms * occ && NG * SC > kRingSpread)
+    k_eval_ring<CG, G><<<grid, C::NT, C::SMEM, st>>>(T, S, s0, offset, Gdev, NG, gsplit, UP, UPq, U, Uq, Wb, M, out,
+                                                     ldo, partial, status);
+  else
+    launch_k(k_eval_ring<CG, G>, grid, dim3(C::NT), C::SMEM, st, T, S, s0, offset, Gdev, NG, gsplit, UP, UPq, U, Uq, Wb,
+             M, out, ldo, partial, status);
   note_launch();
 }
 
 // The instances: columns per consumer and consumer warps for a block of
 // SC <= 64 columns (at most 8 consumers).
-using RingLaunch = void (*)(int64_t, int, int, int, const int64_t*, int64_t, int, const uint64_t*, const uint64_t*,
+using RingLaunch = void (*)(int, int64_t, int, int, int, const int64_t*, int64_t, int, const uint64_t*, const uint64_t*,
                             const uint64_t*,
                             const uint64_t*, const uint64_t*, const Mod&, uint64_t*, int64_t, uint64_t*, uint32_t*,
                             cudaStream_t);
@@ -592,14 +604,14 @@ static int64_t ring_words(int S, int64_t G) {
   return L.off[L.nb - 1] + G * L.bw[L.nb - 1];
 }
 
-static void launch_ring(int64_t T, int S, int offset, const int64_t* Gdev, int64_t NG, int gsplit, const uint64_t* UP,
+static void launch_ring(const zr_ctx* ctx, int64_t T, int S, int offset, const int64_t* Gdev, int64_t NG, int gsplit, const uint64_t* UP,
                         const uint64_t* UPq, const uint64_t* U, const uint64_t* Uq, const uint64_t* Wr,
                         const RingLayout& L, const Mod& M, uint64_t* out, int64_t ldo, uint64_t* partial,
                         uint32_t* status, cudaStream_t st) {
   for (int b = 0; b < L.nb; b++) {
     const int s0 = 64 * b;
     const RingInst* r = ring_inst(S - s0 < 64 ? S - s0 : 64);
-    r->launch(T, S, s0, offset, Gdev, NG, gsplit, UP, UPq, U, Uq, Wr + L.off[b], M, out, ldo, partial, status, st);
+    r->launch(ctx->sms ? ctx->sms : 152, T, S, s0, offset, Gdev, NG, gsplit, UP, UPq, U, Uq, Wr + L.off[b], M, out, ldo, partial, status, st);
   }
 }
 
@@ -820,7 +832,7 @@ zr_status probes_enqueue(zr_ctx* ctx, const zr_poly* f, int k, const uint64_t* y
              w.start, w.cnt, w.order, w.a, f->exps, nv, k, w.tabC, w.U, M, L, rw, nsq, w.Wp, w.UP, w.UPq, w.Uq);
     note_launch();
   }
-  launch_ring(T, S, offset, w.Gdev, Tn, gsplit, w.UP, w.UPq, w.U, w.Uq, w.Wp, L, M, out, ldo, w.partial, status, st);
+  launch_ring(ctx, T, S, offset, w.Gdev, Tn, gsplit, w.UP, w.UPq, w.U, w.Uq, w.Wp, L, M, out, ldo, w.partial, status, st);
   if (gsplit > 1) {
     launch_k(k_eval_combine, dim3(cdiv(T * S, 256)), dim3(256), 0, st, T, S, gsplit, (const int64_t*)nullptr, w.partial, M,
              out, ldo);
