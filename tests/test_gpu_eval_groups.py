@@ -1,5 +1,6 @@
 """GPU parity: the merged weights of groups of several terms, a block and a thread
-per group, for each of the evaluators that read them, against the oracle."""
+per group, for each of the evaluators that read them, and the evaluation of few
+terms at many points, against the oracle."""
 import numpy as np
 import pytest
 
@@ -47,3 +48,14 @@ def test_weights(ctx, orc, G, n, S, T, method):
     sidx, iidx = st.below(40, S), np.concatenate([[0, T - 1], st.below(38, T)])
     want = orc.zippel_probes_sampled(exps, coef, k, y, cs, z, sidx, iidx, offset=1)
     assert np.array_equal(h64(out)[sidx, iidx], want)
+
+
+@pytest.mark.parametrize("Tf", [0, 1, 31, 32, 33])
+@pytest.mark.parametrize("nv,maxexp,npts", [(1, 255, 1217), (5, 20, 1216), (5, 255, 2003), (64, 3, 1500)])
+def test_few_terms_at_many_points(ctx, orc, Tf, nv, maxexp, npts):
+    exps = W.Stream(Tf, 1).below(Tf * nv, maxexp + 1).reshape(Tf, nv).astype(np.uint8)
+    coef, pts = W.Stream(Tf, 2).residues(Tf), W.Stream(npts, 3).residues(npts * nv).reshape(npts, nv)
+    out = zeros64(npts)
+    ke, kc, kp = d8(exps), d64(coef), d64(pts)
+    ctx.eval_points(ctx.poly(nv, Tf, ke, kc), npts, kp, out)
+    assert np.array_equal(h64(out), orc.eval_points(exps, coef, pts))
