@@ -122,6 +122,10 @@ __device__ inline void newton_matrix_warp(int S, const uint64_t* __restrict__ xs
 }
 __device__ __forceinline__ void newton_matrix(int S, const uint64_t* __restrict__ xs_g, uint64_t* W, uint32_t* status,
                                               const Mod& M) {
+  if (S == 1) {                                  // (the inverse of 1 takes as long as any)
+    if ((threadIdx.x & 31) == 0) W[0] = 1;
+    return;
+  }
   if (S <= 32) newton_matrix_warp<1>(S, xs_g, W, status, M);
   else newton_matrix_warp<2>(S, xs_g, W, status, M);
 }
