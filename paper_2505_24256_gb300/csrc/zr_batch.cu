@@ -485,7 +485,7 @@ static bool prepare(const zr_ctx* ctx, const BatchItem* items, int n, Prepared& 
     const BatchItem& it = items[i];
     if (it.mode != P.mode) return false;
     P.fast[i] = use_fast_solve(ctx, it.T, it.solve_S(), n) ? 1 : 0;
-    P.small[i] = !P.fast[i] && small_entry(it.T, it.solve_S(), it.S, it.k) ? 1 : 0;
+    P.small[i] = !P.fast[i] && !it.chain && small_entry(it.T, it.solve_S(), it.S, it.k) ? 1 : 0;
     if (P.small[i]) {
       StepDims D = {};
       D.T = it.T;
@@ -903,6 +903,33 @@ zr_status run_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status
 }
 
 // ---- captured batches (CUDA graphs) ----------------------------------------------
+
+// A small entry is one cluster's chain of dependent steps, and a cluster has its
+// SMs to itself; the kernels of the chain work on all entries at once.  So up to
+// two waves of clusters a call of small entries takes the GPU less time, beyond
+// that the chain does (graph launches, small against chain, S = 1 / 11: 256 of
+// T = 32 50 / 60 against 66 / 75 us, 1024 140 / 172 against 105 / 125; 64 of T =
+// 128 60 / 76 against 79 / 90, 256 195 / 255 against 119 / 155; 16 of T = 200
+// 71 / 90 against 82 / 94, 64 158 / 203 against 107 / 132).  A call that is
+// planned anew each time stays with the small entries: planning the chain costs
+// the host more than the GPU saves (1024 of T = 200, S = 11: 3.8 against 10 ms).
+void plan_repeated(const zr_ctx* ctx, BatchItem* items, int n) {
+  int64_t count = 0, Tmax = 0;
+  size_t words = 0;
+  auto small = [&](const BatchItem& it) {
+    return !it.chain && !use_fast_solve(ctx, it.T, it.solve_S(), n) && small_entry(it.T, it.solve_S(), it.S, it.k);
+  };
+  for (int i = 0; i < n; i++) {
+    const BatchItem& it = items[i];
+    if (!small(it)) continue;
+    count++;
+    Tmax = std::max(Tmax, it.T);
+    words = std::max(words, small_words(it.T, it.solve_S(), it.S, it.k));
+  }
+  if (!count || count <= 2 * (int64_t)small_resident(Tmax, words)) return;
+  for (int i = 0; i < n; i++)
+    if (small(items[i])) items[i].chain = true;
+}
 
 zr_status batch_graph_capture(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, char* ws,
                               cudaStream_t st, cudaGraph_t* graph, uint64_t* launches) {

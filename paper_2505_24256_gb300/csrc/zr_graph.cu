@@ -51,6 +51,7 @@ extern "C" zr_status zr_step_graph_create(zr_ctx* ctx, int32_t nsteps, const zr_
   zr_step_graph* g = new (std::nothrow) zr_step_graph();
   if (!g) return ZR_ERR_OOM;
   g->ctx = ctx;
+  plan_repeated(ctx, items.data(), (int)items.size());
   const size_t need = batch_ws_need(ctx, items.data(), (int)items.size());
   cudaError_t e = cudaMalloc(&g->ws, need > 0 ? need : 256);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_status, sizeof(uint32_t));

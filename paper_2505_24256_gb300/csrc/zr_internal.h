@@ -163,6 +163,7 @@ struct BatchItem {
   // they were taken at).  The step then solves only samples 1..S-1 (b's row
   // 0 is not read) and interpolates through all S.
   const uint64_t* c0 = nullptr;
+  bool chain = false;           // by the chain of kernels, also where it would be a small entry
   int solve_S() const { return c0 && mode == 0 && S >= 2 ? S - 1 : S; }
 };
 // Small entries (zr_small.cu), solved in one launch: whether an entry of T
@@ -170,6 +171,8 @@ struct BatchItem {
 // words it needs, and the launch of the n entries idx[0..n) of Ds.
 bool small_entry(int64_t T, int S, int Sn, int k);
 size_t small_words(int64_t T, int S, int Sn, int k);
+// how many such entries of up to Tmax unknowns and `words` the GPU holds at a time
+int small_resident(int64_t Tmax, size_t words);
 cudaError_t launch_small(const BDesc* Ds, const int64_t* idx, int n, int64_t Tmax, size_t words, const Mod& M,
                          cudaStream_t st);
 // Workspace bytes a batch needs (its regions plus the device tables).
@@ -178,6 +181,9 @@ size_t batch_ws_need(const zr_ctx* ctx, const BatchItem* items, int n);
 // workspace (the caller ensured base + batch_ws_need, or the call grows it
 // when nothing before `base` is live).  status: device word of ST_* flags.
 zr_status run_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, cudaStream_t st, size_t base = 0);
+// Marks the entries of a batch that is run again and again (a graph) `chain`
+// where that takes the GPU less time.
+void plan_repeated(const zr_ctx* ctx, BatchItem* items, int n);
 // The same batch with its workspace at `ws` (batch_ws_need bytes, owned by
 // the caller): the tables are staged and the batch run once on `st`, then its
 // kernels are captured into *graph; *launches counts the captured kernels.

@@ -389,6 +389,27 @@ cudaError_t launch_small(const BDesc* Ds, const int64_t* idx, int n, int64_t Tma
   return e;
 }
 
+int small_resident(int64_t Tmax, size_t words) {
+  const int cl = (int)((Tmax + kSmRoots - 1) / kSmRoots);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cl);
+  cfg.blockDim = dim3(kSmThreads);
+  cfg.dynamicSmemBytes = 8 * words;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_small, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 1;
+  }
+  return clusters > 0 ? clusters : 1;
+}
+
 size_t small_words(int64_t T, int S, int Sn, int k) { return (size_t)small_smem((int)T, S, Sn, k).total; }
 
 }  // namespace zr
