@@ -146,9 +146,10 @@ zr_status zr_measure_peaks(zr_ctx* ctx, zr_peaks* out, void* stream);
  * k-block count): times the `budget` best-ranked candidate plans of that
  * method (whatever zr_solve_method chose) on synthetic data of shape (T, S)
  * and records the fastest in the context; later calls with that shape that
- * take the O(T^2) method use it.  Plans change the schedule only, never the
- * values.
- * zr_step_plan reports the plan a call of shape (T, S) would use. */
+ * take the O(T^2) method's kernels use it (entries of up to 256 unknowns and
+ * 32 samples are one launch without a plan, except in large step graphs).
+ * Plans change the schedule only, never the values.
+ * zr_step_plan reports the plan those kernels would use for shape (T, S). */
 zr_status zr_autotune_step(zr_ctx* ctx, int64_t T, int32_t S, int32_t budget, void* stream);
 zr_status zr_step_plan(zr_ctx* ctx, int64_t T, int32_t S, int32_t* s_tile, int32_t* nblocks);
 

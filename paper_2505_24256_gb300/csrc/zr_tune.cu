@@ -82,6 +82,7 @@ extern "C" zr_status zr_autotune_step(zr_ctx* ctx, int64_t T, int32_t S, int32_t
   it.ldb = T;
   it.c = cc;
   it.ldc = T;
+  it.chain = true;   // the plan is the chain's, also for a shape that calls take in one launch
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);

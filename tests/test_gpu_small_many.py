@@ -1,5 +1,5 @@
 """GPU parity: step graphs of few and of many small entries (one launch, the chain
-of kernels), against the oracle."""
+of kernels), against the oracle; the autotuner at shapes of small entries."""
 import pytest
 
 from tests.pyref import P63
@@ -35,3 +35,14 @@ def test_graph_of_small_entries(ctx, orc, n, sizes, one):
     for d, _, ref in made:                       # (an entry of one sample is all zeros: step)
         check(orc, d, ref)
     g.close()
+
+
+def test_autotuner_times_plans_at_small_shapes(ctx):
+    """Every candidate plan is run (twice) by the kernels it plans, not by the
+    single launch that a small entry is elsewhere."""
+    from paper_2505_24256_gb300 import zr
+
+    before = zr.launch_count()
+    ctx.autotune_step(200, 11, budget=3)
+    assert zr.launch_count() - before >= 3 * 2 * 5
+    assert ctx.step_plan(200, 11)[0] > 0
