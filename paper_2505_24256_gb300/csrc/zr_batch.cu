@@ -709,9 +709,14 @@ static void configure_newton_kernels() {
   });
 }
 
-// Enqueues the batch's kernels on `st` (capturable: no host synchronisation,
-// no allocation).  `prof` records the profiler's phase events.
-static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t st, bool prof) {
+// The branches of a batch that run on other streams: Newton's matrices and the
+// small entries (side), the O(T log^2 T) entries (streams 0 .. fast - 1).
+struct Forks {
+  bool side = false;
+  int fast = 0;
+};
+
+static zr_status launch_kernels(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t st, bool prof, Forks& forks) {
   const Prepared& P = SB.P;
   const int n = SB.n;
   const Mod& M = ctx->M;
@@ -749,6 +754,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       configure_newton_kernels();
       cudaEventRecord(ctx->ev_fork, st);
       cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
+      forks.side = true;
       if (mode == 0) {
         launch_k(k_b_newton_table, n, 32, 0, ctx->side, dD, M);
         note_launch();
@@ -790,6 +796,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
     if (!ok) return cuda_err(ctx, cudaErrorMemoryAllocation, "fast streams");
     cudaEventRecord(ctx->fev_fork, st);
     for (int j = 0; j < P.fstreams; j++) cudaStreamWaitEvent(ctx->fstream[j], ctx->fev_fork, 0);
+    forks.fast = P.fstreams;
     int k = 0;
     for (int i = 0; i < n; i++) {
       if (!P.fast[i]) continue;
@@ -851,6 +858,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       if (r) return r;
     }
   for (int j = 0; j < fs_used; j++) cudaStreamWaitEvent(st, ctx->fev_join[j], 0);
+  forks.fast = 0;
   cudaEvent_t e4f = mark();
   // a6 (or the plain finish of a system)
   if (nroots) {
@@ -871,6 +879,7 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
       { launch_k(k_b_finish_solve, cdiv(nroots, 256), 256, 0, st, dD, dpre + o_roots, n, M); note_launch(); }
       if (side) cudaStreamWaitEvent(st, ctx->ev_join, 0);   // the small entries (forked above)
     }
+    forks.side = false;
   }
   cudaEvent_t e5 = mark();
   if (mode == 0 && nroots) {
@@ -889,6 +898,21 @@ static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t s
   prof_add(ctx, PH_NEWTON, e4f, e5);
   prof_add(ctx, PH_COMPACT, e5, e6);
   return cuda_err(ctx, cudaGetLastError(), "batch launch");
+}
+
+// Enqueues the batch's kernels on `st` (capturable: no host synchronisation,
+// no allocation).  `prof` records the profiler's phase events.  Where a part
+// cannot be enqueued, `st` waits for the branches that are under way: they read
+// the tables and write the workspace that the next call lays out anew.
+static zr_status launch_batch(zr_ctx* ctx, const StagedBatch& SB, cudaStream_t st, bool prof) {
+  Forks forks;
+  const zr_status r = launch_kernels(ctx, SB, st, prof, forks);
+  auto join = [&](cudaEvent_t e, cudaStream_t from) {
+    if (cudaEventRecord(e, from) == cudaSuccess) cudaStreamWaitEvent(st, e, 0);
+  };
+  if (forks.side) join(ctx->ev_join, ctx->side);
+  for (int j = 0; j < forks.fast; j++) join(ctx->fev_join[j], ctx->fstream[j]);
+  return r;
 }
 
 zr_status run_batch(zr_ctx* ctx, const BatchItem* items, int n, uint32_t* status, cudaStream_t st, size_t base) {
