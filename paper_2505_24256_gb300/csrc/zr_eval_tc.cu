@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kEtcThreads, 1)
 #pragma unroll
       for (int c = 0; c < 16; c++) acc[c] = TcAcc{{0, 0, 0, 0, 0, 0}};
       for (int k = 0; k < n; k += kEtcChunkSteps, ph ^= 1) {
-        if (!mbar_wait(tfull, ph)) {
+        if (!tc_wait(tfull, ph)) {
           atomicOr(status, ST_TIMEOUT);
           ok = false;
           break;
@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(kEtcThreads, 1)
         const int st = t % kEtcStages;
         const bool first = k % kEtcChunkSteps == 0, last = k % kEtcChunkSteps == kEtcChunkSteps - 1 || k == n - 1;
         const uint32_t ph = (t / kEtcStages) & 1;
-        if ((first && ch > 0 && !mbar_wait(tempty, (ch - 1) & 1)) || !mbar_wait(&fullA[st], ph) ||
-            !mbar_wait(&fullB[st], ph)) {
+        if ((first && ch > 0 && !tc_wait(tempty, (ch - 1) & 1)) || !tc_wait(&fullA[st], ph) ||
+            !tc_wait(&fullB[st], ph)) {
           if (leader) atomicOr(status, ST_TIMEOUT);
           ok = false;
           break;
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kEtcThreads, 1)
         load(k + 2);
         uint4 d[kTcLimbs];
         tc_digits(x, M.p, d);
-        if (tt >= kEtcStages && !mbar_wait(&empty[st], ((tt / kEtcStages) & 1) ^ 1)) {
+        if (tt >= kEtcStages && !tc_wait(&empty[st], ((tt / kEtcStages) & 1) ^ 1)) {
           atomicOr(status, ST_TIMEOUT);
           ok = false;
           break;

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kLfThreads, 2)
     bool ok = true;
     int drained = 0;
     auto drain = [&]() {
-      if (!mbar_wait(tfull, drained & 1)) {
+      if (!tc_wait(tfull, drained & 1)) {
         atomicOr(status, ST_TIMEOUT);
         ok = false;
         return;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kLfThreads, 2)
     for (int s = 0; ok && s < n; s++) {
       const int st = s % kLfStages;
       uint4* dst = reinterpret_cast<uint4*>(lsm + st * kLfStage) + 32 * warp + lane;
-      if (s >= kLfStages && !mbar_wait(&empty[st], ((s / kLfStages) & 1) ^ 1)) {
+      if (s >= kLfStages && !tc_wait(&empty[st], ((s / kLfStages) & 1) ^ 1)) {
         atomicOr(status, ST_TIMEOUT);
         ok = false;
         break;
@@ -142,7 +142,10 @@ __global__ void __launch_bounds__(kLfThreads, 2)
       if (s + 1 >= kLfChunkSteps + kLfAhead && (s + 1 - kLfAhead) % kLfChunkSteps == 0) drain();
     }
     while (ok && drained < chunks) drain();
-    if (ok && !mbar_wait(summed, 0)) ok = false;
+    if (ok && !tc_wait(summed, 0)) {
+      atomicOr(status, ST_TIMEOUT);
+      ok = false;
+    }
     if (ok && live) {
 #pragma unroll
       for (int c = 0; c < kLfNC; c++) {
@@ -174,7 +177,7 @@ __global__ void __launch_bounds__(kLfThreads, 2)
       for (int i = 0; i < 8; i++) sum = add_mod(sum, x[i], M);
       tc_digits(x, M.p, dg);
       load(s + 1);
-      if (s >= kLfStages && !mbar_wait(&empty[st], ((s / kLfStages) & 1) ^ 1)) {
+      if (s >= kLfStages && !tc_wait(&empty[st], ((s / kLfStages) & 1) ^ 1)) {
         atomicOr(status, ST_TIMEOUT);
         break;
       }
@@ -195,7 +198,7 @@ __global__ void __launch_bounds__(kLfThreads, 2)
     for (int s = 0; s < n; s++) {
       const int st = s % kLfStages, c = s / kLfChunkSteps;
       const bool first = s % kLfChunkSteps == 0, last = s % kLfChunkSteps == kLfChunkSteps - 1 || s == n - 1;
-      if ((first && c > 0 && !mbar_wait(tempty, (c - 1) & 1)) || !mbar_wait(&full[st], (s / kLfStages) & 1)) {
+      if ((first && c > 0 && !tc_wait(tempty, (c - 1) & 1)) || !tc_wait(&full[st], (s / kLfStages) & 1)) {
         if (leader) atomicOr(status, ST_TIMEOUT);
         break;
       }

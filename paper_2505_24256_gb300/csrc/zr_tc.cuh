@@ -80,6 +80,11 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 // generic-proxy writes to shared memory before the tensor core reads them
 __device__ __forceinline__ void tc_fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// A bounded wait of a whole warp: its lanes go on, or give up, together (the
+// instructions behind it are the warp's).
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
 // one lane of a converged warp
 __device__ __forceinline__ bool tc_elect() {
   uint32_t r;
