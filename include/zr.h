@@ -358,6 +358,12 @@ zr_status zr_zippel_step_host(zr_ctx* ctx, const zr_poly* skel, int32_t newvar, 
 zr_status zr_zippel_probes(zr_ctx* ctx, const zr_poly* f, int32_t k, const uint64_t* y, int32_t S,
                            const uint64_t* samples, const uint64_t* z, int64_t T, int32_t offset, uint64_t* out,
                            int64_t ldo, void* stream);
+/* The evaluator a call of T probes per sample of Tf terms takes, as
+ * zr_step_plan does for the solve: *method 0 the integer kernel, 1 the tensor
+ * cores, 2 the transposed tree (above 2^18 terms the number of groups may still
+ * send it to the integer kernel); *splits the parts the terms are divided into
+ * (0 for the tree).  Either may be NULL. */
+zr_status zr_probe_plan(const zr_ctx* ctx, int64_t T, int64_t Tf, int32_t S, int32_t* method, int32_t* splits);
 /* f at npts arbitrary points (device, npts x nv). */
 zr_status zr_eval_points(zr_ctx* ctx, const zr_poly* f, int64_t npts, const uint64_t* pts, uint64_t* out,
                          void* stream);

@@ -1014,6 +1014,17 @@ extern "C" zr_status zr_zippel_probes(zr_ctx* ctx, const zr_poly* f, int32_t k, 
   return status_from_flags(ctx, ctx->h_status[1]);
 }
 
+extern "C" zr_status zr_probe_plan(const zr_ctx* ctx, int64_t T, int64_t Tf, int32_t S, int32_t* method,
+                                   int32_t* splits) {
+  if (!ctx || T < 1 || Tf < 1 || S < 1 || S > 256) return ZR_ERR_INVALID_ARG;
+  const EvalMethod m = eval_method(ctx, T, Tf, S);
+  Carver cv(nullptr);
+  if (method) *method = m;
+  if (splits)
+    *splits = m == EVAL_TREE ? 0 : m == EVAL_TC ? carve_eval_tc(cv, ctx, Tf, S, T).gsplit : eval_gsplit(ctx, T, S, Tf);
+  return ZR_OK;
+}
+
 extern "C" zr_status zr_eval_points(zr_ctx* ctx, const zr_poly* f, int64_t npts, const uint64_t* pts, uint64_t* out,
                                     void* stream) {
   if (!ctx) return ZR_ERR_INVALID_ARG;

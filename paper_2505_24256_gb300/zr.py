@@ -109,6 +109,7 @@ SIGNATURES = {
     "zr_profile_work": (_ST, [_V, _I32, ctypes.POINTER(ctypes.c_double)]),
     "zr_autotune_step": (_ST, [_V, _I64, _I32, _I32, _V]),
     "zr_step_plan": (_ST, [_V, _I64, _I32, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
+    "zr_probe_plan": (_ST, [_V, _I64, _I64, _I32, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
     "zr_solve_method": (_ST, [_V, _I32, _I64]),
     "zr_vandermonde_solve_batched": (_ST, [_V, _I32, _P, _V]),
     "zr_vandermonde_solve_plain": (_ST, [_V, _I32, _P, _V]),
@@ -296,6 +297,14 @@ class Context:
         tile, nb = ctypes.c_int32(), ctypes.c_int32()
         self.check(self.L.zr_step_plan(self._h, T, S, ctypes.byref(tile), ctypes.byref(nb)), "zr_step_plan")
         return tile.value, nb.value
+
+    PROBE_RING, PROBE_TC, PROBE_TREE = 0, 1, 2
+
+    def probe_plan(self, T, Tf, S):
+        """The evaluator (PROBE_*) and its splits for T probes per sample of Tf terms."""
+        method, splits = ctypes.c_int32(), ctypes.c_int32()
+        self.check(self.L.zr_probe_plan(self._h, T, Tf, S, ctypes.byref(method), ctypes.byref(splits)), "zr_probe_plan")
+        return method.value, splits.value
 
     def profile_query(self, phase):
         idx = self.PHASES.index(phase) if isinstance(phase, str) else int(phase)
