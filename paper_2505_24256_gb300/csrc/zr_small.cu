@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(kSmThreads, 1)
   __shared__ uint64_t sq[kMaxVars][8], rs[kSmWarps][kSmRoots], us[kSmWarps][kSmRoots], invs[kSmRoots];
   __shared__ uint32_t nz[32], masks[kSmRoots];
   __shared__ int offs[kSmRoots], tot[8];
+  asm volatile("barrier.cluster.arrive;" ::: "memory");   // waited for before another CTA's memory is written
   const int ent = blockIdx.x / cl, rank = blockIdx.x - ent * cl;
   const BDesc& D = Ds[idx[ent]];
-  if (D.mode == 0) asm volatile("barrier.cluster.arrive;" ::: "memory");   // waited for before another CTA's memory is written
   const int T = (int)D.T, S = D.S, Sn = D.Sn, k = D.mode == 0 ? D.k : 0, s1 = Sn - S;
   const SmallSmem o = small_smem(T, S, Sn, k);
   uint64_t *vs = ssm + o.v, *tree = ssm + o.tree, *tab = ssm + o.tab, *bs = ssm + o.b, *qs = ssm + o.q,
@@ -248,7 +248,9 @@ __global__ void __launch_bounds__(kSmThreads, 1)
   }
   __syncthreads();
   // every CTA has read all the nodes: a system's solution may lie over them
-  if (D.mode != 0) asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+  // (the arrival at the top is an early one: a barrier of its own)
+  if (D.mode != 0)
+    asm volatile("barrier.cluster.wait;\n\tbarrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
   if (any && warp < kSmWarps) {
     const uint64_t inv = invs[lane];
     if (D.mode != 0) {
