@@ -484,8 +484,8 @@ def fast_roofline(ctx, peaks, workload_name, steps, step_ms):
         entries.append((ms, {
             "bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gop/s",
             "frac": achieved / peak,
-            "traffic": kernel_traffic(kernel, workload_name, NTT_SOURCES), "traffic_unit": "bytes/launch",
-            "kernel": kernel, "ops": ops,
+            "traffic": kernel_traffic(kernel.split(",")[0], workload_name, NTT_SOURCES),
+            "traffic_unit": "bytes/launch", "kernel": kernel, "ops": ops,
             "launch_ms": ms / n, "share_of_step": ms / max(steps, 1) / step_ms,
             "peak_basis": basis}))
     if not entries:

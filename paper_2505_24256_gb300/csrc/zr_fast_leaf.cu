@@ -40,7 +40,7 @@ constexpr uint32_t kLfTmem = 256;
 // each step waiting for the one before).  The blocks of 128 roots on the integer
 // pipe, a thread per root that ran its chain again for every four rows, took
 // 0.040 ms at T = 10^4, S = 21 and 1.31 ms at T = 2^20, S = 9; this kernel takes
-// 0.048 and 1.32 ms for blocks of 256 (0.35 ms at T = 125000, S = 9), which saves
+// 0.048 and 1.32 ms for blocks of 256 (0.18 ms at T = 125000, S = 9), which saves
 // the descent's level of 2^8 (0.040 and 1.6 ms).
 __global__ void __launch_bounds__(kLfThreads, 2)
     k_leaf_tc(const uint64_t* __restrict__ coef, const uint64_t* __restrict__ X, int R, int cols, int ll, int64_t T,
