@@ -160,7 +160,8 @@ zr_status zr_step_plan(zr_ctx* ctx, int64_t T, int32_t S, int32_t* s_tile, int32
  *     offset 0:  sum_j c[s][j] v_j^k     = b[s][k],  k = 0..T-1
  *     offset 1:  sum_j c[s][j] v_j^(k+1) = b[s][k],  k = 0..T-1
  *   T       number of unknowns (>= 0)
- *   S       right-hand sides (1..256)
+ *   S       right-hand sides (1..256; above 64 only where the O(T log^2 T)
+ *           method takes the system, else ZR_ERR_INVALID_ARG)
  *   v       device, T nodes (pairwise distinct; nonzero when offset = 1)
  *   b       device, S x ldb (ldb >= T)
  *   c       device, S x ldc output (ldc >= T); may not alias b
